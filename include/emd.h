@@ -164,7 +164,7 @@ typedef struct {
     int64_t launches[EMD_N_PHASES];
     int64_t total_launches; /* every kernel launch since creation, profiling on or off */
     int64_t pruned_queries; /* max-direction top-K queries answered by the pruned path */
-    int64_t prune_fallbacks; /* of those, queries recomputed over all documents */
+    int64_t prune_fallbacks; /* of those, queries that needed the second stage (see emd_topk) */
     int64_t graph_launches;  /* batch sequences replayed from captured graphs (their kernels are
                                 included in the launch counts) */
     int64_t ict_wide;        /* ICT queries recomputed with tables of full width h because a
@@ -221,10 +221,12 @@ emd_status emd_query_batch(emd_db* db, const emd_queries* q, emd_measure meas, i
 /* The K nearest database histograms of each query (Section 6, top-l neighbours), in
  * ascending (distance, document id) order.
  * For EMD_DIR_MAX with K <= 16 (and prune_topk set) the reverse direction is evaluated
- * only where it can matter: max(fwd, rev) >= fwd, so the documents are taken in ascending
- * forward order, the reverse pass runs on the 63 best, and the answer is certified when the
- * K-th symmetric value is strictly below the 64th forward value; a query that fails the
- * test is recomputed over all documents.  The result equals the unpruned one.
+ * only where it can matter: max(fwd, rev) >= fwd, so the reverse pass runs on the documents
+ * within a margin of the K-th smallest forward value (at most 256), and the answer is
+ * certified when the K-th symmetric value does not exceed that margin.  For a query that
+ * fails the test the K-th symmetric value U found so far still bounds the answer, and a second
+ * stage evaluates every document with a forward value <= U.  The result equals the unpruned
+ * one.
  *   K         1..min(n_docs, 256)
  *   out_idx   host int64 [n_queries * K]; out_dist host float [n_queries * K]
  * Otherwise as emd_query_batch. */

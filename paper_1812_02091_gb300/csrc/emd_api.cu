@@ -326,6 +326,16 @@ emd_status run_lanes(emd_db* db, const int64_t* rp, const int32_t* qidx, const f
                      int64_t i1, int meas, int k, int dir, int K, bool pruned, float* out_t, int64_t* out_idx,
                      float* out_dist, cudaStream_t st);
 
+// Whether a sub-batch runs in the fused form (the Phase-1 table from the product's epilogue,
+// reverse distances on the candidate documents' rows only).
+bool fused_form(const BatchWS& ws, const emd_db* db, int meas, int k, int dir, bool pruned, bool allow_fused)
+{
+    if (!pruned || !allow_fused || !ws.fused || meas == M_ICT) return false;
+    const int H = db->opt.max_query_h;
+    const int tk_b = dir != EMD_DIR_REV ? table_width(db, meas, k, H) : 0;
+    return tk_b <= 16 && (!db->approx || std::min(rerank_width(db, tk_b, H), kRerankMax) <= kCandPerRow);
+}
+
 // The kernels of one sub-batch whose descriptors sit in ring slot `slot`.  Grids are sized
 // from bounds (qcap queries, max_query_h bins, the table width of k) and every block checks
 // the query count on the device, so the same sequence serves every batch of at most qcap
@@ -341,8 +351,7 @@ emd_status launch_sequence(BatchWS& ws, emd_db* db, int slot, int meas, int k, i
     const int H = db->opt.max_query_h;
     const int tk_b = dir != EMD_DIR_REV ? table_width(db, meas, k, H) : 0;
     const int kc_b = db->approx ? std::min(rerank_width(db, tk_b, H), kRerankMax) : tk_b;
-    if (pruned && allow_fused && ws.fused && !hd && meas != M_ICT && tk_b <= 16 &&
-        (!db->approx || kc_b <= kCandPerRow)) {
+    if (!hd && fused_form(ws, db, meas, k, dir, pruned, allow_fused)) {
         // fused form: the table from the product's epilogue (approximate formats: candidates
         // re-ranked exactly); the reverse direction's distances on the candidate documents' rows
         // only, exact in the FP16 split
@@ -634,9 +643,9 @@ void free_batch_ws(BatchWS& ws)
 // batch fits the batch workspace) and uploads them on st.  Outputs as run_batch.
 emd_status fill_descriptors(BatchWS& ws, int slot, emd_db* db, const int64_t* rp, const int32_t* qidx, const float* qw, int64_t i0,
                         int64_t j0, int64_t j1, int meas, int k, int dir, int K, bool pruned, float* out_t,
-                        int64_t* out_idx, float* out_dist, cudaStream_t st)
+                        int64_t* out_idx, float* out_dist, cudaStream_t st, const std::vector<int64_t>* pick = nullptr)
 {
-    const int nb = (int)(j1 - j0);
+    const int nb = pick ? (int)pick->size() : (int)(j1 - j0);
     const int tk_b = dir != EMD_DIR_REV ? table_width(db, meas, k, db->opt.max_query_h) : 0;
     const bool grouped = grouped_tables(ws, meas, tk_b);
     const int lw_b = grouped_width(db, meas, tk_b);
@@ -653,7 +662,7 @@ emd_status fill_descriptors(BatchWS& ws, int slot, emd_db* db, const int64_t* rp
     // Every output is addressed per query (b = i - i0), so results do not depend on the order.
     std::vector<int64_t>& order = ws.order;
     order.resize((size_t)nb);
-    for (int p = 0; p < nb; ++p) order[p] = j0 + p;
+    for (int p = 0; p < nb; ++p) order[p] = pick ? (*pick)[(size_t)p] : j0 + p;
     if (grouped)
         std::stable_sort(order.begin(), order.end(),
                          [&](int64_t x, int64_t y) { return rp[x + 1] - rp[x] > rp[y + 1] - rp[y]; });
@@ -792,47 +801,16 @@ emd_status run_subbatch_launch(BatchWS& ws, int slot, emd_db* db, int nb, int me
     return EMD_OK;
 }
 
-// Ring slots are reused only after the work that reads them (pinned host copy and device
-// descriptors) has finished, whatever stream it ran on.
-emd_status run_subbatch(emd_db* db, BatchWS& ws, const int64_t* rp, const int32_t* qidx, const float* qw, int64_t i0,
-                        int64_t j0, int64_t j1, int meas, int k, int dir, int K, bool pruned, float* out_t,
-                        int64_t* out_idx, float* out_dist, cudaStream_t st, bool allow_fused)
-{
-    const int slot = ws.desc_slot;
-    ws.desc_slot = (slot + 1) % BatchWS::kDescRing;
-    EMD_CUDA(cudaEventSynchronize(ws.desc_ev[slot]), "descriptor ring");
-    if (meas == M_ICT)
-        EMD_CUDA(cudaMemsetAsync(ws.ict_over + (j0 - i0), 0, (j1 - j0) * sizeof(int), st), "flag reset");
-    emd_status s = fill_descriptors(ws, slot, db, rp, qidx, qw, i0, j0, j1, meas, k, dir, K, pruned, out_t, out_idx,
-                                    out_dist, st);
-    if (s == EMD_OK) s = run_subbatch_launch(ws, slot, db, (int)(j1 - j0), meas, k, dir, K, pruned, st, allow_fused);
-    EMD_CUDA(cudaEventRecord(ws.desc_ev[slot], st), "descriptor ring");
-    return s;
-}
-
-emd_status retry_materialized(emd_db* db, BatchWS& ws, const int64_t* rp, const int32_t* qidx, const float* qw,
-                              int64_t i0, int64_t i, int meas, int k, int K, int64_t* out_idx, float* out_dist,
-                              cudaStream_t st, int* ok)
-{
-    const int64_t off = rp[i] - rp[i0];
-    // a sub-batch of its own: query i with offsets relative to itself, outputs at row i - i0
-    const int64_t rp1[2] = {0, rp[i + 1] - rp[i]};
-    emd_status s = run_subbatch(db, ws, rp1, qidx + off, qw + off, 0, 0, 1, meas, k, EMD_DIR_MAX, K, true, nullptr,
-                                out_idx + (i - i0) * K, out_dist + (i - i0) * K, st, false);
-    if (s != EMD_OK) return s;
-    EMD_CUDA(cudaMemcpyAsync(ok, ws.cand_ok, sizeof(int), cudaMemcpyDeviceToHost, st), "flag read");
-    EMD_CUDA(cudaStreamSynchronize(st), "synchronize");
-    return EMD_OK;
-}
-
-bool batch_fits(const emd_db* db, const BatchWS& ws, const int64_t* rp, int64_t i0, int64_t i1, int meas, int k,
-                int dir)
+// Whether the queries ids[0..count) (ids null: i0..i0+count-1) fit one sub-batch of ws.
+bool list_fits(const emd_db* db, const BatchWS& ws, const int64_t* rp, const int64_t* ids, int64_t count, int meas, int k,
+               int dir, int64_t i0 = 0)
 {
     int64_t cD = 0, cQ = 0, cP = 0, cT = 0;
-    if (i1 - i0 > ws.max_batch) return false;
+    if (count > ws.max_batch) return false;
     const int tk_b = dir != EMD_DIR_REV ? table_width(db, meas, k, db->opt.max_query_h) : 0;
     const bool grouped = grouped_tables(ws, meas, tk_b);
-    for (int64_t i = i0; i < i1; ++i) {
+    for (int64_t t = 0; t < count; ++t) {
+        const int64_t i = ids ? ids[t] : i0 + t;
         const int h = (int)(rp[i + 1] - rp[i]);
         const int64_t ldd = round_up(h, 32);
         cD += ldd;
@@ -842,9 +820,102 @@ bool batch_fits(const emd_db* db, const BatchWS& ws, const int64_t* rp, int64_t 
     }
     if (grouped) {  // whole groups of kFwdGroup tables
         const int lw = grouped_width(db, meas, tk_b);
-        cT = (i1 - i0 + kFwdGroup - 1) / kFwdGroup * kFwdGroup * (lw ? lw : tk_b);
+        cT = (count + kFwdGroup - 1) / kFwdGroup * kFwdGroup * (lw ? lw : tk_b);
     }
     return cD <= ws.b_cols && cQ <= ws.b_qrows && cP <= ws.b_prows && cT <= ws.b_tabcols;
+}
+
+bool batch_fits(const emd_db* db, const BatchWS& ws, const int64_t* rp, int64_t i0, int64_t i1, int meas, int k,
+                int dir)
+{
+    return list_fits(db, ws, rp, nullptr, i1 - i0, meas, k, dir, i0);
+}
+
+// Ring slots are reused only after the work that reads them (pinned host copy and device
+// descriptors) has finished, whatever stream it ran on.
+emd_status run_subbatch(emd_db* db, BatchWS& ws, const int64_t* rp, const int32_t* qidx, const float* qw, int64_t i0,
+                        int64_t j0, int64_t j1, int meas, int k, int dir, int K, bool pruned, float* out_t,
+                        int64_t* out_idx, float* out_dist, cudaStream_t st, bool allow_fused,
+                        const std::vector<int64_t>* pick)
+{
+    const int slot = ws.desc_slot;
+    ws.desc_slot = (slot + 1) % BatchWS::kDescRing;
+    EMD_CUDA(cudaEventSynchronize(ws.desc_ev[slot]), "descriptor ring");
+    if (meas == M_ICT && !pick)
+        EMD_CUDA(cudaMemsetAsync(ws.ict_over + (j0 - i0), 0, (j1 - j0) * sizeof(int), st), "flag reset");
+    const int nb = pick ? (int)pick->size() : (int)(j1 - j0);
+    emd_status s = fill_descriptors(ws, slot, db, rp, qidx, qw, i0, j0, j1, meas, k, dir, K, pruned, out_t, out_idx,
+                                    out_dist, st, pick);
+    if (s == EMD_OK) s = run_subbatch_launch(ws, slot, db, nb, meas, k, dir, K, pruned, st, allow_fused);
+    ws.last_slot = slot;
+    ws.last_dense = !fused_form(ws, db, meas, k, dir, pruned, allow_fused);
+    ws.last_j0 = pick ? 0 : j0;
+    ws.last_j1 = pick ? 0 : j1;
+    EMD_CUDA(cudaEventRecord(ws.desc_ev[slot], st), "descriptor ring");
+    return s;
+}
+
+// The second stage of the pruned top-K on the queries of the last sub-batch (ring slot
+// ws.last_slot, nb queries, full distance matrices in place).
+emd_status second_stage(emd_db* db, BatchWS& ws, int nb, int meas, int k, int K, cudaStream_t st)
+{
+    const QDesc* D_ = ws.qd_dev + (int64_t)ws.last_slot * ws.max_batch;
+    const int* nqd = ws.nq_dev + ws.last_slot;
+    {
+        Phase p(db, 4, 1, st);
+        EMD_CUDA(launch_rev_within_b(meas, k, D_, nqd, nb, db->row_ptr, db->col, db->val, db->n, K, st),
+                 "reverse pass (second stage)");
+    }
+    {
+        Phase p(db, 5, topk_launch_count(db->n), st);
+        EMD_CUDA(launch_topk_b(D_, nqd, nb, db->n, K, ws.topk_scratch, false, st, true), "top-K (second stage)");
+    }
+    EMD_CUDA(cudaEventRecord(ws.desc_ev[ws.last_slot], st), "descriptor ring");
+    return EMD_OK;
+}
+
+emd_status resolve_uncertified(emd_db* db, BatchWS& ws, const int64_t* rp, const int32_t* qidx, const float* qw,
+                               int64_t i0, int64_t i1, int meas, int k, int K, int64_t* out_idx, float* out_dist,
+                               cudaStream_t st, int* ok, const int* over, int64_t* uncertified)
+{
+    *uncertified = 0;
+    bool in_place = false;
+    std::vector<int64_t> todo;
+    for (int64_t i = i0; i < i1; ++i) {
+        if (ok[i - i0] == 1 || (over && over[i - i0])) continue;
+        if (ok[i - i0] == 2) ++db->fused_retries; else ++*uncertified;
+        if (ws.last_dense && i >= ws.last_j0 && i < ws.last_j1) in_place = true; else todo.push_back(i);
+    }
+    if (in_place) {
+        emd_status s = second_stage(db, ws, (int)(ws.last_j1 - ws.last_j0), meas, k, K, st);
+        if (s != EMD_OK) return s;
+    }
+    // the others: once more with the full matrix, as many at a time as the workspace holds
+    std::vector<int64_t> pick;
+    std::vector<int> flags((size_t)(i1 - i0), 1);
+    for (size_t t = 0; t < todo.size();) {
+        pick.clear();
+        bool retried = false;
+        do {
+            retried |= ok[todo[t] - i0] == 2;
+            pick.push_back(todo[t++]);
+        } while (t < todo.size() && list_fits(db, ws, rp, todo.data() + (t - pick.size()), (int64_t)pick.size() + 1, meas,
+                                              k, EMD_DIR_MAX));
+        emd_status s = run_subbatch(db, ws, rp, qidx, qw, i0, 0, 0, meas, k, EMD_DIR_MAX, K, true, nullptr, out_idx,
+                                    out_dist, st, false, &pick);
+        if (s == EMD_OK) s = second_stage(db, ws, (int)pick.size(), meas, k, K, st);
+        if (s != EMD_OK) return s;
+        if (!retried) continue;
+        EMD_CUDA(cudaMemcpyAsync(flags.data(), ws.cand_ok, (size_t)(i1 - i0) * sizeof(int), cudaMemcpyDeviceToHost, st),
+                 "flag read");
+        EMD_CUDA(cudaStreamSynchronize(st), "synchronize");
+        for (int64_t i : pick)
+            if (ok[i - i0] == 2) {
+                ok[i - i0] = flags[(size_t)(i - i0)];
+                *uncertified += ok[i - i0] != 1;
+            }
+    }
+    return EMD_OK;
 }
 
 emd_status run_batch(emd_db* db, const int64_t* rp, const int32_t* qidx, const float* qw, int64_t i0,
@@ -875,8 +946,8 @@ emd_status run_batch(emd_db* db, const int64_t* rp, const int32_t* qidx, const f
         }
     }
     if (!pruned && !ict) return EMD_OK;
-    // uncertified pruned queries and ICT queries whose table overflowed: recomputed alone
-    // over all documents (ICT with tables of full width)
+    // uncertified pruned queries: the second stage (batched form) or a run over all documents;
+    // ICT queries whose table overflowed: recomputed alone with tables of full width
     std::vector<int> ok((size_t)(i1 - i0), 1), over((size_t)(i1 - i0), 0);
     if (pruned)
         EMD_CUDA(cudaMemcpyAsync(ok.data(), db->opt.batched ? db->bw.cand_ok : db->cand_ok, (i1 - i0) * sizeof(int),
@@ -888,13 +959,15 @@ emd_status run_batch(emd_db* db, const int64_t* rp, const int32_t* qidx, const f
                  "flag read");
     EMD_CUDA(cudaStreamSynchronize(st), "synchronize");
     if (pruned) db->pruned_queries += i1 - i0;
+    if (pruned && db->opt.batched) {
+        int64_t uncertified = 0;
+        emd_status s = resolve_uncertified(db, db->bw, rp, qidx, qw, i0, i1, meas, k, K, out_idx, out_dist, st,
+                                           ok.data(), over.data(), &uncertified);
+        if (s != EMD_OK) return s;
+        db->prune_fallbacks += uncertified;
+        ok.assign(ok.size(), 1);
+    }
     for (int64_t i = i0; i < i1; ++i) {
-        if (db->opt.batched && pruned && ok[i - i0] == 2) {  // the fused candidate block overflowed
-            ++db->fused_retries;
-            emd_status s = retry_materialized(db, db->bw, rp, qidx, qw, i0, i, meas, k, K, out_idx, out_dist, st,
-                                              &ok[i - i0]);
-            if (s != EMD_OK) return s;
-        }
         if (ok[i - i0] == 1 && !over[i - i0]) continue;
         if (over[i - i0]) ++db->ict_wide; else ++db->prune_fallbacks;
         const int64_t off = rp[i] - rp[i0];

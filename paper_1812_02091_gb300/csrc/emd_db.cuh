@@ -123,6 +123,11 @@ struct BatchWS {
     int* nq_host = nullptr;
     cudaEvent_t desc_ev[kDescRing] = {};
     int desc_slot = 0;
+    // the last sub-batch run on this workspace: its ring slot and query range, and whether its
+    // full distance matrices are still in bD (not the fused form)
+    int last_slot = 0;
+    bool last_dense = false;
+    int64_t last_j0 = 0, last_j1 = 0;
     cudaStream_t cap_stream = nullptr;  // graph capture
     std::map<GraphKey, GraphEntry> graphs;
 };
@@ -290,15 +295,21 @@ void free_batch_ws(BatchWS& ws);
 // Sub-batch j0..j1-1 of the queries i0.. (host rp, device qidx / qw relative to query i0)
 // on ws, in ring slot order: descriptors, then the batched sequence (graph replay when
 // enabled) on st.  Outputs: out_t rows (K = 0), else out_idx / out_dist rows, relative to
-// i0; certification flags in ws.cand_ok[i - i0] on the pruned path.  Caller holds db->mu.
+// i0; certification flags in ws.cand_ok[i - i0] on the pruned path.  pick: these queries
+// instead of j0..j1-1.  Caller holds db->mu.
 emd_status run_subbatch(emd_db* db, BatchWS& ws, const int64_t* rp, const int32_t* qidx, const float* qw,
                         int64_t i0, int64_t j0, int64_t j1, int meas, int k, int dir, int K, bool pruned,
-                        float* out_t, int64_t* out_idx, float* out_dist, cudaStream_t st, bool allow_fused = true);
-// Pruned query i (of the batch starting at i0) whose fused candidate block overflowed: run
-// again alone on ws with the full distance matrix; *ok receives its new certification flag.
-emd_status retry_materialized(emd_db* db, BatchWS& ws, const int64_t* rp, const int32_t* qidx, const float* qw,
-                              int64_t i0, int64_t i, int meas, int k, int K, int64_t* out_idx, float* out_dist,
-                              cudaStream_t st, int* ok);
+                        float* out_t, int64_t* out_idx, float* out_dist, cudaStream_t st, bool allow_fused = true,
+                        const std::vector<int64_t>* pick = nullptr);
+// Completes a pruned batch i0..i1-1 run on ws from its certification flags ok[i - i0] (host
+// copies; 0 not certified, 2 the fused candidate block overflowed): queries that are not
+// certified get the second stage (k_rev_within_b) on the distance matrices of the last
+// sub-batch where these are still in place, else after a run with the full matrix.  Queries
+// with over[i - i0] (ICT tables cut short; may be null) are left alone.  ok receives the
+// final flags; *uncertified the number of queries the second stage answered.
+emd_status resolve_uncertified(emd_db* db, BatchWS& ws, const int64_t* rp, const int32_t* qidx, const float* qw,
+                               int64_t i0, int64_t i1, int meas, int k, int K, int64_t* out_idx, float* out_dist,
+                               cudaStream_t st, int* ok, const int* over, int64_t* uncertified);
 // Whether the batch (rp entries i0..i1) fits one sub-batch of ws.
 bool batch_fits(const emd_db* db, const BatchWS& ws, const int64_t* rp, int64_t i0, int64_t i1, int meas, int k,
                 int dir);

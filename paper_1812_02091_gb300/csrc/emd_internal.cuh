@@ -334,8 +334,14 @@ cudaError_t launch_rev_b(int meas, int k, int dir, const QDesc* qd, const int* n
 // Top-K of each query of a batch: from t_fwd into sel_idx / sel_val (fwd_rows: the
 // forward top-K of the pruned path) or from t_out into out_idx / out_dist.  scratch holds
 // max_q * kTopkScratchRow keys.
+// uncertified: only the queries whose certification flag is not 1.
 cudaError_t launch_topk_b(const QDesc* qd, const int* nq, int max_q, int64_t n, int K,
-                          unsigned long long* scratch, bool fwd_rows, cudaStream_t st);
+                          unsigned long long* scratch, bool fwd_rows, cudaStream_t st, bool uncertified = false);
+// Second stage of the pruned top-K for the batch's uncertified queries (their D, t_fwd and first
+// K symmetric values still in place): t_out = max(fwd, rev) of the documents that can still
+// enter, +inf elsewhere.
+cudaError_t launch_rev_within_b(int meas, int k, const QDesc* qd, const int* nq, int nb, const int32_t* row_ptr,
+                                const int32_t* col, const float* val, int64_t n, int K, cudaStream_t st);
 // Pruned top-K after the forward top-K (sel_idx / sel_val): candidate compaction (counts
 // must be zeroed), reverse pass on the candidates, final selection and certificate.
 // rev_warps: warps per candidate document in the reverse pass (2, 4 or 8; same results).

@@ -205,58 +205,59 @@ emd_status launch_batch(emd_server* s, Exec& e)
     return EMD_OK;
 }
 
-// Recomputes over all documents, in place in the pinned results, the batch's uncertified
-// pruned requests and its ICT requests whose table overflowed (both rare; ICT with tables of
-// full width); *count receives how many.
+// Completes, in place in the pinned results, the batch's uncertified pruned requests (second
+// stage over the documents that can still enter) and its ICT requests whose table overflowed
+// (recomputed over all documents with tables of full width), both rare; *count receives how
+// many.
 emd_status run_fallbacks(emd_server* s, Exec& e, int* count)
 {
     emd_db* db = s->db;
     *count = 0;
     const bool ict = ict_batch(db, e);
     if (!e.pruned && !ict) return EMD_OK;
-    for (size_t i = 0; i < e.batch.size(); ++i) {
+    const int nb = (int)e.batch.size();
+    std::vector<char> redo((size_t)nb, 0);
+    bool any = false, resolve = false;
+    for (int i = 0; i < nb; ++i) {
         const bool over = ict && e.h_over[i];
-        const Request* r = e.batch[i];
-        if (!over && e.pruned && e.h_ok[i] == 2) {  // the fused candidate block overflowed
-            {
-                std::lock_guard<std::mutex> lock(db->mu);
-                ++db->fused_retries;
-                emd_status st = retry_materialized(db, e.ws, e.h_rp, e.d_idx, e.d_w, 0, (int64_t)i, r->meas, r->k,
-                                                   r->K, e.d_oidx, e.d_odist, e.st, &e.h_ok[i]);
-                if (st != EMD_OK) return st;
-            }
-            if (e.h_ok[i] == 1) {
-                EMD_CUDA(cudaMemcpyAsync(e.h_oidx + i * r->K, e.d_oidx + i * r->K, (size_t)r->K * 8,
-                                         cudaMemcpyDeviceToHost, e.st),
-                         "result copy");
-                EMD_CUDA(cudaMemcpyAsync(e.h_odist + i * r->K, e.d_odist + i * r->K, (size_t)r->K * 4,
-                                         cudaMemcpyDeviceToHost, e.st),
-                         "result copy");
-                EMD_CUDA(cudaStreamSynchronize(e.st), "synchronize");
-                continue;
-            }
+        redo[(size_t)i] = over || (e.pruned && e.h_ok[i] != 1);
+        any |= redo[(size_t)i] != 0;
+        resolve |= !over && e.pruned && e.h_ok[i] != 1;
+    }
+    if (!any) return EMD_OK;
+    {
+        std::lock_guard<std::mutex> lock(db->mu);
+        if (resolve) {
+            int64_t uncertified = 0;
+            emd_status st = resolve_uncertified(db, e.ws, e.h_rp, e.d_idx, e.d_w, 0, nb, e.meas, e.k, e.K, e.d_oidx,
+                                                e.d_odist, e.st, e.h_ok, ict ? e.h_over : nullptr, &uncertified);
+            if (st != EMD_OK) return st;
+            db->prune_fallbacks += uncertified;
+            *count += (int)uncertified;
         }
-        if (!over && (!e.pruned || e.h_ok[i] == 1)) continue;
-        const int64_t off = e.h_rp[i];
-        {
-            std::lock_guard<std::mutex> lock(db->mu);
+        for (int i = 0; i < nb; ++i) {
+            if (!(ict && e.h_over[i])) continue;
+            const Request* r = e.batch[(size_t)i];
+            const int64_t off = e.h_rp[i];
             emd_status st = run_query(db, s->fb, e.d_idx + off, e.d_w + off, r->h, r->meas, r->k, EMD_DIR_MAX,
                                       s->fb_out, nullptr, e.st);
             if (st != EMD_OK) return st;
-            EMD_CUDA(launch_topk(s->fb_out, db->n, r->K, s->fb.scratch, e.d_oidx + i * r->K, e.d_odist + i * r->K,
-                                 e.st),
+            EMD_CUDA(launch_topk(s->fb_out, db->n, r->K, s->fb.scratch, e.d_oidx + (int64_t)i * r->K,
+                                 e.d_odist + (int64_t)i * r->K, e.st),
                      "top-K");
-            if (over) db->ict_wide += 1; else db->prune_fallbacks += 1;
+            db->ict_wide += 1;
+            ++*count;
         }
-        EMD_CUDA(cudaMemcpyAsync(e.h_oidx + i * r->K, e.d_oidx + i * r->K, (size_t)r->K * 8, cudaMemcpyDeviceToHost,
-                                 e.st),
-                 "result copy");
-        EMD_CUDA(cudaMemcpyAsync(e.h_odist + i * r->K, e.d_odist + i * r->K, (size_t)r->K * 4,
-                                 cudaMemcpyDeviceToHost, e.st),
-                 "result copy");
-        EMD_CUDA(cudaStreamSynchronize(e.st), "synchronize");
-        ++*count;
     }
+    for (int i = 0; i < nb; ++i) {
+        if (!redo[(size_t)i]) continue;
+        const int64_t o = (int64_t)i * e.K;
+        EMD_CUDA(cudaMemcpyAsync(e.h_oidx + o, e.d_oidx + o, (size_t)e.K * 8, cudaMemcpyDeviceToHost, e.st),
+                 "result copy");
+        EMD_CUDA(cudaMemcpyAsync(e.h_odist + o, e.d_odist + o, (size_t)e.K * 4, cudaMemcpyDeviceToHost, e.st),
+                 "result copy");
+    }
+    EMD_CUDA(cudaStreamSynchronize(e.st), "synchronize");
     return EMD_OK;
 }
 

@@ -41,12 +41,12 @@ cudaError_t launch_cand_rows_b(const QDesc* qd, const int* nq, int max_q, const 
 
 
 cudaError_t launch_topk_b(const QDesc* qd, const int* nq, int max_q, int64_t n, int K,
-                          unsigned long long* scratch, bool fwd_rows, cudaStream_t st)
+                          unsigned long long* scratch, bool fwd_rows, cudaStream_t st, bool uncertified)
 {
     if (max_q <= 0) return cudaSuccess;
-    if (K <= 16) return topk_kt_b<16>(qd, nq, max_q, n, K, scratch, fwd_rows, st);
-    if (K <= 32) return topk_kt_b<32>(qd, nq, max_q, n, K, scratch, fwd_rows, st);
-    return topk_kt_b<64>(qd, nq, max_q, n, K, scratch, fwd_rows, st);
+    if (K <= 16) return topk_kt_b<16>(qd, nq, max_q, n, K, scratch, fwd_rows, uncertified, st);
+    if (K <= 32) return topk_kt_b<32>(qd, nq, max_q, n, K, scratch, fwd_rows, uncertified, st);
+    return topk_kt_b<64>(qd, nq, max_q, n, K, scratch, fwd_rows, uncertified, st);
 }
 
 }  // namespace emd
