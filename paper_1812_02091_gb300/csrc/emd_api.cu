@@ -98,9 +98,6 @@ cudaEvent_t take_event(emd_db* db)
     return e;
 }
 
-// Whether a batch's forward tables are interleaved in groups of kFwdGroup queries (one CSR
-// sweep per group): register-width tables, and ICT tables (the loop form) when a group of
-// them fits the workspace's table columns.
 // The fused FP32_TC table runs on SM pairs when the option asks for it and the panel fits.
 bool use_tc_pair(const emd_db* db)
 {
@@ -108,10 +105,37 @@ bool use_tc_pair(const emd_db* db)
            tc_table_pair_fits(db->kpad);
 }
 
-bool grouped_tables(const BatchWS& ws, int meas, int tk_b)
+// Size class of a sub-batch of nb queries: what its grids (and its graph) cover.
+int batch_qcap(const BatchWS& ws, int64_t nb)
 {
-    return tk_b > 0 && (tk_b <= 16 || (meas == M_ICT && (int64_t)kFwdGroup * tk_b <= ws.b_tabcols));
+    int qcap = 1;
+    while (qcap < nb) qcap *= 2;
+    return std::min(qcap, ws.max_batch);
 }
+
+// Whether grouped tables of width tk_b are swept by the entry-chain form: when it is the form in
+// use, and for the wide ICT tables that the vector-load forms do not take.
+bool chain_form(const emd_db* db, int tk_b)
+{
+    return db->tune_fwd == kFwdChain || (db->tune_fwd != kFwdPrefetch && fwd_reg_width(tk_b) == 0);
+}
+
+// Queries per interleaved group of forward tables (one CSR sweep per group) in a sub-batch of
+// size class qcap, 0 when its tables are not interleaved: register-width tables, and ICT tables
+// (the loop form) when a group of them fits the workspace's table columns.
+int table_group(const emd_db* db, const BatchWS& ws, int meas, int tk_b, int qcap)
+{
+    const int64_t w = chain_form(db, tk_b) ? round_up(tk_b, 2) : tk_b;  // room for pairs
+    if (tk_b <= 0 || !(tk_b <= 16 || (meas == M_ICT && kFwdGroup * w <= ws.b_tabcols))) return 0;
+    if (!chain_form(db, tk_b)) return kFwdGroup;
+    const int g = fwd_chain_group(qcap, tk_b);
+    return g * w <= ws.b_tabcols ? g : kFwdGroup;
+}
+
+// Whether a sub-batch's grouped tables hold their entries in adjacent pairs, and the entries of
+// a row in the layout (the entry-chain form from width 2 on).
+bool paired_tables(const emd_db* db, int tk_b) { return chain_form(db, tk_b) && tk_b >= 2; }
+int layout_width(const emd_db* db, int tk_b) { return paired_tables(db, tk_b) ? (tk_b + 1) / 2 * 2 : tk_b; }
 
 // Row width of a query's table in the grouped, query-major layout (the forward kernel's
 // register width), or 0 for the entry-interleaved layout of wide ICT tables.
@@ -397,8 +421,8 @@ emd_status launch_sequence(BatchWS& ws, emd_db* db, int slot, int meas, int k, i
         }
         {
             Phase p(db, 3, 1, st);
-            EMD_CUDA(launch_fwd_b(meas, D_, nqd, B, db->row_ptr, db->col, db->val, n, false,
-                                  grouped_tables(ws, meas, tk_b), tk_b, st, db->tune_fwd),
+            EMD_CUDA(launch_fwd_b(meas, D_, nqd, B, db->row_ptr, db->col, db->val, db->sweep, n, false,
+                                  table_group(db, ws, meas, tk_b, B), tk_b, st, db->tune_fwd),
                      "forward pass");
         }
         {
@@ -479,8 +503,8 @@ emd_status launch_sequence(BatchWS& ws, emd_db* db, int slot, int meas, int k, i
                          "top-k table");
         }
         Phase p(db, 3, 1, st);
-        EMD_CUDA(launch_fwd_b(meas, D_, nqd, B, db->row_ptr, db->col, db->val, n, dir == EMD_DIR_FWD,
-                              grouped_tables(ws, meas, tk_b), tk_b, st, db->tune_fwd),
+        EMD_CUDA(launch_fwd_b(meas, D_, nqd, B, db->row_ptr, db->col, db->val, db->sweep, n, dir == EMD_DIR_FWD,
+                              table_group(db, ws, meas, tk_b, B), tk_b, st, db->tune_fwd),
                  "forward pass");
     }
     if (pruned) {
@@ -565,7 +589,7 @@ emd_status alloc_batch_ws(emd_db* db, BatchWS& ws, int max_batch, int64_t cols, 
     ws.b_cols = std::max<int64_t>(round_up(cols, 32), round_up(db->opt.max_query_h, 32));
     ws.b_qrows = ws.b_cols + 32 * B;
     ws.b_prows = ws.b_cols + 96 * B;
-    ws.b_tabcols = std::max<int64_t>(db->opt.max_table_k, 16 * round_up(B, kFwdGroup));  // whole interleaved groups
+    ws.b_tabcols = std::max<int64_t>(db->opt.max_table_k, 16 * round_up(B, kFwdGroupMax));  // whole interleaved groups
     TRYW(dal(&ws.bD, vu * ws.b_cols));
     if (!db->cost_mode) {
         TRYW(dal(&ws.bQ, ws.b_qrows * db->ldm));
@@ -641,13 +665,14 @@ void free_batch_ws(BatchWS& ws)
 
 // Fills ring slot `slot` with the descriptors of queries j0..j1-1 of the batch i0.. (the
 // batch fits the batch workspace) and uploads them on st.  Outputs as run_batch.
-emd_status fill_descriptors(BatchWS& ws, int slot, emd_db* db, const int64_t* rp, const int32_t* qidx, const float* qw, int64_t i0,
+emd_status fill_descriptors(BatchWS& ws, int slot, int qcap, emd_db* db, const int64_t* rp, const int32_t* qidx, const float* qw, int64_t i0,
                         int64_t j0, int64_t j1, int meas, int k, int dir, int K, bool pruned, float* out_t,
                         int64_t* out_idx, float* out_dist, cudaStream_t st, const std::vector<int64_t>* pick = nullptr)
 {
     const int nb = pick ? (int)pick->size() : (int)(j1 - j0);
     const int tk_b = dir != EMD_DIR_REV ? table_width(db, meas, k, db->opt.max_query_h) : 0;
-    const bool grouped = grouped_tables(ws, meas, tk_b);
+    const int grp = table_group(db, ws, meas, tk_b, qcap);
+    const bool grouped = grp > 0;
     const int lw_b = grouped_width(db, meas, tk_b);
     QDesc* hd = ws.qd_host + (int64_t)slot * ws.max_batch;
     QDesc* dd = ws.qd_dev + (int64_t)slot * ws.max_batch;
@@ -656,7 +681,7 @@ emd_status fill_descriptors(BatchWS& ws, int slot, emd_db* db, const int64_t* rp
     int max_rows = 0, max_npad = 0, max_ldd = 0, max_tk = 0, max_kc = 0;
     int64_t c_D = 0, c_Q = 0, c_P = 0, c_T = 0;
     // Descriptor position p holds query order[p].  With grouped tables the forward sweep runs
-    // a group of kFwdGroup consecutive positions in one warp, whose lanes step through the
+    // a group of consecutive positions in one warp, whose lanes step through the
     // longest transfer chain of the group (longer for larger h_q, whose capacities are
     // smaller), so the queries are placed by h_q, largest first: groups of alike lengths.
     // Every output is addressed per query (b = i - i0), so results do not depend on the order.
@@ -697,9 +722,11 @@ emd_status fill_descriptors(BatchWS& ws, int slot, emd_db* db, const int64_t* rp
             d.tab_es = 1;
         } else if (grouped) {
             const int64_t bs = p;
-            d.tab = ws.btab + (bs / kFwdGroup) * (db->v_used * tk_b * kFwdGroup) + bs % kFwdGroup;
-            d.tab_rs = tk_b * kFwdGroup;
-            d.tab_es = kFwdGroup;
+            const int w = layout_width(db, tk_b), pair = paired_tables(db, tk_b) ? 1 : 0;
+            d.tab = ws.btab + (bs / grp) * (db->v_used * w * grp) + ((bs % grp) << pair);
+            d.tab_rs = w * grp;
+            d.tab_es = grp << pair;
+            d.tab_pair = pair;
         } else {
             d.tab = ws.btab + c_T * db->v_used;
             d.tab_rs = d.tk;
@@ -758,7 +785,7 @@ emd_status fill_descriptors(BatchWS& ws, int slot, emd_db* db, const int64_t* rp
         max_kc = std::max(max_kc, d.kc);
     }
     // the caller sizes sub-batches with batch_fits; never let one overrun the workspace
-    const int64_t tab_used = grouped ? (int64_t)(nb + kFwdGroup - 1) / kFwdGroup * kFwdGroup * (lw_b ? lw_b : tk_b) : c_T;
+    const int64_t tab_used = grouped ? (int64_t)(nb + grp - 1) / grp * grp * (lw_b ? lw_b : layout_width(db, tk_b)) : c_T;
     if (nb > ws.max_batch || c_D > ws.b_cols || c_Q > ws.b_qrows || c_P > ws.b_prows || tab_used > ws.b_tabcols)
         return fail(EMD_ERR_INVALID_ARG, "internal: sub-batch of %d queries exceeds the batch workspace", nb);
     ws.nq_host[slot] = nb;
@@ -773,9 +800,7 @@ emd_status run_subbatch_launch(BatchWS& ws, int slot, emd_db* db, int nb, int me
                                cudaStream_t st, bool allow_fused)
 {
     const QDesc* hd = ws.qd_host + (int64_t)slot * ws.max_batch;
-    int qcap = 1;  // size class of the batch: the next power of two
-    while (qcap < nb) qcap *= 2;
-    qcap = std::min(qcap, ws.max_batch);
+    const int qcap = batch_qcap(ws, nb);
     if (db->tc && tc_batch_stages(db->tcfmt, db->kpad / 64) < 2) {
         // embeddings too wide for the batched panel: Phase 1 per query, the rest batched
         return launch_sequence(ws, db, slot, meas, k, K, dir, pruned, hd, nb, qcap, st);
@@ -808,7 +833,7 @@ bool list_fits(const emd_db* db, const BatchWS& ws, const int64_t* rp, const int
     int64_t cD = 0, cQ = 0, cP = 0, cT = 0;
     if (count > ws.max_batch) return false;
     const int tk_b = dir != EMD_DIR_REV ? table_width(db, meas, k, db->opt.max_query_h) : 0;
-    const bool grouped = grouped_tables(ws, meas, tk_b);
+    const int grp = table_group(db, ws, meas, tk_b, batch_qcap(ws, count));
     for (int64_t t = 0; t < count; ++t) {
         const int64_t i = ids ? ids[t] : i0 + t;
         const int h = (int)(rp[i + 1] - rp[i]);
@@ -818,9 +843,9 @@ bool list_fits(const emd_db* db, const BatchWS& ws, const int64_t* rp, const int
         cP += round_up(h, 128);
         cT += dir != EMD_DIR_REV ? table_width(db, meas, k, h) : 0;
     }
-    if (grouped) {  // whole groups of kFwdGroup tables
+    if (grp > 0) {  // whole groups of tables
         const int lw = grouped_width(db, meas, tk_b);
-        cT = (count + kFwdGroup - 1) / kFwdGroup * kFwdGroup * (lw ? lw : tk_b);
+        cT = (count + grp - 1) / grp * grp * (lw ? lw : layout_width(db, tk_b));
     }
     return cD <= ws.b_cols && cQ <= ws.b_qrows && cP <= ws.b_prows && cT <= ws.b_tabcols;
 }
@@ -844,7 +869,7 @@ emd_status run_subbatch(emd_db* db, BatchWS& ws, const int64_t* rp, const int32_
     if (meas == M_ICT && !pick)
         EMD_CUDA(cudaMemsetAsync(ws.ict_over + (j0 - i0), 0, (j1 - j0) * sizeof(int), st), "flag reset");
     const int nb = pick ? (int)pick->size() : (int)(j1 - j0);
-    emd_status s = fill_descriptors(ws, slot, db, rp, qidx, qw, i0, j0, j1, meas, k, dir, K, pruned, out_t, out_idx,
+    emd_status s = fill_descriptors(ws, slot, batch_qcap(ws, nb), db, rp, qidx, qw, i0, j0, j1, meas, k, dir, K, pruned, out_t, out_idx,
                                     out_dist, st, pick);
     if (s == EMD_OK) s = run_subbatch_launch(ws, slot, db, nb, meas, k, dir, K, pruned, st, allow_fused);
     ws.last_slot = slot;
@@ -1104,7 +1129,7 @@ emd_status autotune(emd_db* db, const std::vector<int32_t>& used_host)
     EMD_CUDA(cudaMemcpyAsync(db->stage_idx, idx.data(), idx.size() * 4, cudaMemcpyHostToDevice, st), "tune copy");
     EMD_CUDA(cudaMemcpyAsync(db->stage_w, w.data(), w.size() * 4, cudaMemcpyHostToDevice, st), "tune copy");
     const bool pruned = prunable(db, EMD_ACT, k, EMD_DIR_MAX, K);
-    emd_status s = fill_descriptors(ws, 0, db, rp.data(), db->stage_idx, db->stage_w, 0, 0, nb, EMD_ACT, k, EMD_DIR_MAX, K,
+    emd_status s = fill_descriptors(ws, 0, ws.max_batch, db, rp.data(), db->stage_idx, db->stage_w, 0, 0, nb, EMD_ACT, k, EMD_DIR_MAX, K,
                                     pruned, nullptr, db->stage_oidx, db->stage_odist, st);
     if (s != EMD_OK) return s;
     const bool per_query_tc = db->tc && tc_batch_stages(db->tcfmt, db->kpad / 64) < 2;
@@ -1177,7 +1202,7 @@ emd_status autotune(emd_db* db, const std::vector<int32_t>& used_host)
         int choice = kFwdChain;
         for (int v : {kFwdChain, kFwdPrefetch, kFwdCoalesced, kFwdRowMajor}) {
             db->tune_fwd = v;
-            s = fill_descriptors(ws, 0, db, rp.data(), db->stage_idx, db->stage_w, 0, 0, nb, EMD_ACT, k, EMD_DIR_MAX,
+            s = fill_descriptors(ws, 0, ws.max_batch, db, rp.data(), db->stage_idx, db->stage_w, 0, 0, nb, EMD_ACT, k, EMD_DIR_MAX,
                                  K, pruned, nullptr, db->stage_oidx, db->stage_odist, st);
             if (s == EMD_OK)
                 s = launch_sequence(ws, db, 0, EMD_ACT, k, K, EMD_DIR_MAX, pruned, per_query_tc ? ws.qd_host : nullptr,
@@ -1185,8 +1210,8 @@ emd_status autotune(emd_db* db, const std::vector<int32_t>& used_host)
             if (s != EMD_OK) return s;
             const int tk = table_width(db, EMD_ACT, k, db->opt.max_query_h);
             const float ms = timed([&] {
-                launch_fwd_b(EMD_ACT, D_, nqd, db->opt.max_batch, db->row_ptr, db->col, db->val, db->n, false,
-                             grouped_tables(ws, EMD_ACT, tk), tk, st, v);
+                launch_fwd_b(EMD_ACT, D_, nqd, db->opt.max_batch, db->row_ptr, db->col, db->val, db->sweep, db->n, false,
+                             table_group(db, ws, EMD_ACT, tk, ws.max_batch), tk, st, v);
             });
             if (ms < 0.95f * best) {
                 best = ms;
@@ -1340,6 +1365,7 @@ emd_status emd_db_create(const float* emb, int64_t v, int32_t m, const float* co
     TRY(dalloc(db, &db->row_ptr, n_docs + 1));
     TRY(dalloc(db, &db->col, nnz));
     TRY(dalloc(db, &db->val, nnz));
+    TRY(dalloc(db, &db->cv, nnz));
     TRY(dalloc(db, &db->err, 1));
     TRYC(cudaMemsetAsync(db->err, 0, sizeof(int), st), "memset");
     TRYC(cudaMemcpyAsync(db->used_ids, used_ids.data(), vu * sizeof(int32_t), cudaMemcpyHostToDevice, st), "copy");
@@ -1350,6 +1376,26 @@ emd_status emd_db_create(const float* emb, int64_t v, int32_t m, const float* co
     TRYC(cudaMemcpyAsync(db->row_ptr, rp32.data(), (n_docs + 1) * sizeof(int32_t), cudaMemcpyHostToDevice, st), "copy");
     TRYC(cudaMemcpyAsync(db->col, col_used.data(), nnz * sizeof(int32_t), cudaMemcpyHostToDevice, st), "copy");
     TRYC(cudaMemcpyAsync(db->val, val, nnz * sizeof(float), cudaMemcpyHostToDevice, st), "copy");
+    TRYC(launch_interleave(db->col, db->val, nnz, db->cv, st), "CSR pairs");
+    {
+        // documents past twice the mean length, longest first (at least 32: below, a document is
+        // one or two steps of the sweep)
+        const int64_t lim = std::max<int64_t>(32, 2 * nnz / n_docs);
+        std::vector<int32_t> longs;
+        for (int64_t d = 0; d < n_docs; ++d)
+            if (row_ptr[d + 1] - row_ptr[d] > lim) longs.push_back((int32_t)d);
+        std::sort(longs.begin(), longs.end(), [&](int32_t x, int32_t y) {
+            const int64_t hx = row_ptr[x + 1] - row_ptr[x], hy = row_ptr[y + 1] - row_ptr[y];
+            return hx != hy ? hx > hy : x < y;
+        });
+        int32_t* dl = nullptr;
+        TRY(dalloc(db, &dl, (int64_t)longs.size()));
+        if (!longs.empty())
+            TRYC(cudaMemcpy(dl, longs.data(), longs.size() * sizeof(int32_t), cudaMemcpyHostToDevice), "copy");
+        db->sweep = FwdSweep{db->cv, dl, (int)longs.size(), (int)std::min<int64_t>(lim, INT32_MAX)};
+    }
+    db->total_launches += 1;
+    db->launches[6] += 1;
     {
         // the largest weight any document puts on each used row: how far an ICT table row
         // must reach (Algorithm 2 moves at most that much mass out of a bin of the row)

@@ -152,6 +152,8 @@ struct emd_db {
     std::vector<int64_t> row_ptr_host;  // the same offsets on the host (all-pairs batching)
     int32_t* col = nullptr;      // nnz, renumbered into the used vocabulary
     float* val = nullptr;        // nnz
+    int2* cv = nullptr;          // nnz, (col, val) interleaved for the forward sweep
+    emd::FwdSweep sweep;         // cv and the long documents, as the sweep takes them
     int* err = nullptr;
 
     // tensor-core operands of the used vocabulary (precisions FP32_TC, BF16, FP8_E4M3)

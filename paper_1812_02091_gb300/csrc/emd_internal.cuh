@@ -194,7 +194,9 @@ struct QDesc {
     int64_t* out_idx;       // K top-K result
     float* out_dist;
     int h, ldd, qrows, npad, tk, kc;
-    int tab_rs, tab_es;     // table layout: entry l of row u at tab[u * tab_rs + l * tab_es]
+    // table layout: entry l of row u at tab[u * tab_rs + tab_entry(d, l)] -- tab_es apart, or (pairs)
+    // two entries adjacent and the pairs tab_es apart
+    int tab_rs, tab_es, tab_pair;
     // fused form of the pruned path (Phase-1 table in the product's epilogue, no full matrix)
     int32_t* qpos;          // v_used: the query bin whose vocabulary id is used row u, else -1
     int32_t* rmap;          // v_used: row of used row u in the candidate block, else -1
@@ -219,6 +221,18 @@ struct QDesc {
     int* rr_count;
 };
 
+__device__ __forceinline__ int64_t tab_entry(int l, int es, int pair)
+{
+    return (int64_t)(l >> pair) * es + (l & pair);
+}
+
+// Capacity stored with entry l of a row of tk entries: the query bin's weight; in the paired
+// layout the last entry's is +inf, since it takes whatever mass is left.
+__device__ __forceinline__ float tab_cap(float w, int l, int tk, int pair)
+{
+    return pair && l == tk - 1 ? __int_as_float(0x7f800000) : w;
+}
+
 // Candidate bins kept per vocabulary row by the fused approximate forms (k + margin <= 16).
 constexpr int kCandPerRow = 16;
 
@@ -227,12 +241,24 @@ constexpr int kCandPerRow = 16;
 // recomputed over all documents with the full distance matrix).
 constexpr int kCandRows = 32768;
 
-// Queries whose forward pass shares one sweep of the CSR (batched form).  Tables of width
-// <= 16 are stored query-major within a row -- row u, query g, entry l at
-// base[(u * kFwdGroup + g) * W + l] with W the register width of the table (1, 2, 4, 8 or
-// 16) -- so that a lane reads its query's first entries with vector loads; ICT tables of
-// other widths are interleaved by entry, base[(u * width + l) * kFwdGroup + g].
+// Queries whose forward pass shares one sweep of the CSR (batched form).  The entry-chain form
+// (the default) takes 1, 2, 4, 8 or 16 queries a group by the batch's size class, the other
+// forms always kFwdGroup.  Tables are interleaved by entry -- row u, entry l, query g of a group of
+// G at base[(u * width + l) * G + g] -- and in the entry-chain form, from width 2 on, by pairs of
+// entries: base[(u * width + (l & ~1)) * G + 2 g + (l & 1)], width rounded up to even; the query-major form stores tables of width <= 16
+// query-major within a row -- row u, query g, entry l at base[(u * kFwdGroup + g) * W + l]
+// with W the register width of the table (1, 2, 4, 8 or 16).
 constexpr int kFwdGroup = 8;
+constexpr int kFwdGroupMax = 16;
+// Group size of the entry-chain form for tables of width tk in a batch whose grids cover qcap
+// queries: the smallest power of two that holds them (lanes of absent queries would idle), up
+// to the group whose load of a table row is one full 128-byte line -- 8 queries of paired
+// entries, 16 of single ones.
+__host__ __device__ inline int fwd_chain_group(int qcap, int tk)
+{
+    const int most = tk >= 2 ? 8 : 16;
+    return qcap <= 1 ? 1 : qcap <= 2 ? 2 : qcap <= 4 ? 4 : qcap <= 8 ? 8 : most;
+}
 __host__ __device__ inline int fwd_reg_width(int kw)
 {
     return kw <= 1 ? 1 : kw <= 2 ? 2 : kw <= 4 ? 4 : kw <= 8 ? 8 : kw <= 16 ? 16 : 0;
@@ -315,8 +341,8 @@ cudaError_t launch_table_b(const QDesc* qd, const int* nq, int max_q, int64_t M,
 // The ICT table of every query of a batch (width qd[q].tk, overflow flag qd[q].over).
 cudaError_t launch_table_ict_b(const QDesc* qd, const int* nq, int max_q, int64_t M, const float* xmax,
                                cudaStream_t st);
-// Forward values into t_out (to_out) or t_fwd.  grouped: the tables are interleaved in
-// groups of kFwdGroup queries and each group shares one sweep of the CSR.  variant: the form
+// Forward values into t_out (to_out) or t_fwd.  group > 0: the tables are interleaved in
+// groups of that many queries and each group shares one sweep of the CSR.  variant: the form
 // of the grouped sweep (same values for each; the grouped table layout follows it, see
 // fwd_layout_rowmajor):
 //   kFwdChain     entry-interleaved rows, each entry loaded once the residual needs it
@@ -324,9 +350,18 @@ cudaError_t launch_table_ict_b(const QDesc* qd, const int* nq, int max_q, int64_
 //   kFwdCoalesced entry-interleaved rows, the first two entries up front, coalesced CSR reads
 //   kFwdPrefetch  the entry chain with each lane's next four column ids and weights read ahead
 enum : int { kFwdChain = 0, kFwdRowMajor = 1, kFwdCoalesced = 2, kFwdPrefetch = 3, kFwdVariants = 4 };
+// What the entry-chain sweep reads beside row_ptr, made once per database: the CSR as (column,
+// weight bits) pairs, and the documents of more than long_len nonzeros, longest first.
+struct FwdSweep {
+    const int2* cv = nullptr;
+    const int32_t* long_docs = nullptr;
+    int n_long = 0, long_len = 0;
+};
 cudaError_t launch_fwd_b(int meas, const QDesc* qd, const int* nq, int max_q, const int32_t* row_ptr,
-                         const int32_t* col, const float* val, int64_t n, bool to_out, bool grouped, int max_tk,
-                         cudaStream_t st, int variant);
+                         const int32_t* col, const float* val, const FwdSweep& sweep, int64_t n, bool to_out,
+                         int group, int max_tk, cudaStream_t st, int variant);
+// cv[e] = (col[e], val[e] as float bits).
+cudaError_t launch_interleave(const int32_t* col, const float* val, int64_t nnz, int2* cv, cudaStream_t st);
 // Reverse pass over all documents; dir FWD is not accepted, REV writes t_out, MAX writes
 // t_rev and max(t_fwd, t_rev) into t_out.
 cudaError_t launch_rev_b(int meas, int k, int dir, const QDesc* qd, const int* nq, int max_q,

@@ -116,6 +116,16 @@ __global__ void k_fwd(const int32_t* __restrict__ row_ptr, const int32_t* __rest
 
 // ------------------------------------------------------------------ batched forms
 
+// Shape of the entry-chain sweep: blocks of two warps; nonzeros in flight per position (UN) and
+// resident blocks per SM (the register bound).  Groups of up to 4 queries have few warps to
+// run and take more nonzeros each; paired tables at 32 blocks (all 64 warps) and two
+// nonzeros beat 16 to 24 blocks with up to four (serving database, 64 queries: 9.9 against
+// 10.5 to 13.1 ms, a few spilled registers included); single-entry tables are fastest at 24
+// blocks and three.
+constexpr int kFwdThreads = 64;
+constexpr int fwd_un(int meas, int kt, int g) { return g <= 4 ? 4 : meas == M_RWMD || kt == 1 ? 3 : 2; }
+constexpr int fwd_blocks(int meas, int kt, int g) { return g <= 4 ? 16 : meas == M_RWMD || kt == 1 ? 24 : 32; }
+
 template <int MEAS, int KT>
 __global__ void k_fwd_b(const QDesc* __restrict__ qd, const int* __restrict__ nq, const int32_t* __restrict__ row_ptr,
                         const int32_t* __restrict__ col, const float* __restrict__ val, int64_t n, bool to_out)
@@ -125,52 +135,153 @@ __global__ void k_fwd_b(const QDesc* __restrict__ qd, const int* __restrict__ nq
     fwd_body<MEAS, KT>(row_ptr, col, val, n, d.tab, d.tk, d.tk, to_out ? d.t_out : d.t_fwd);
 }
 
-// One sweep of the CSR for a group of kFwdGroup (8) consecutive queries of the batch: a warp
-// takes a document, lane = 8 x phase + query.  The 8 lanes of a nonzero read the same col /
-// val and adjacent table entries (the group's tables are interleaved by entry), so a gather
-// instruction touches 4 table rows instead of 32; the CSR is read once per group.  Values
-// are bit-identical to the per-query form (same phases, same order).  The sweep is bound by
-// the latency of its dependent gathers, not by bandwidth: 32 registers give 8 blocks (all 64
-// warps) per SM, and two nonzeros per lane per step fit in them (four spill or cost occupancy;
-// measured on 1e6 documents, 64 mixed-size queries: 19.6 ms at 6 blocks and four nonzeros,
-// 16.9 ms at 8 blocks and two).
-template <int MEAS, int KT>
-__global__ void __launch_bounds__(256, 8)
-k_fwd_g(const QDesc* __restrict__ qd, const int* __restrict__ nq, const int32_t* __restrict__ row_ptr,
-        const int32_t* __restrict__ col, const float* __restrict__ val, int64_t n, bool to_out)
+// Costs of U nonzeros (weights r, table rows T; a weight of 0 costs nothing and is not
+// gathered) from rows stored in pairs of entries (z0, w0, z1, w1), pairs es4 float4 apart, the
+// last entry's capacity stored as +inf: the steps of fwd_cost_s in the same order (the last
+// entry takes the rest: fmaf(min(r, inf), z, c) is its fmaf(r, z, c)), so bit-identical.  A
+// pair comes with one load, only while mass remains, and the U loads are issued before their
+// arithmetic: one trip to the cache for two entries of U nonzeros.  The warp leaves once no lane
+// has mass left.  width_max: the entries to walk, the same for every lane (the warp votes in
+// the loop): KT, or for KT = 0 (rows wider than 16) the largest width of the warp.  Called by
+// full warps.
+template <int MEAS, int KT, int U>
+__device__ __forceinline__ void fwd_cost_pairs(float (&r)[U], const float4* const (&T)[U], int es4, int width_max,
+                                               float (&c)[U])
 {
-    const int q0 = blockIdx.y * kFwdGroup;
+    float4 t[U];
+    if (MEAS == M_OMR) {
+#pragma unroll
+        for (int j = 0; j < U; ++j)
+            if (r[j] != 0.f) t[j] = T[j][0];
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+            c[j] = 0.f;
+            if (r[j] != 0.f) {
+                // one-bin queries: the only entry's capacity is +inf and takes everything, at cost x z0
+                const float m = r[j] - fminf(r[j], t[j].y);  // after the free transfer to the overlapping bin
+                c[j] = t[j].x != 0.f ? __fmul_rn(r[j], t[j].x) : m != 0.f ? __fmul_rn(m, t[j].z) : 0.f;
+            }
+        }
+        return;
+    }
+#pragma unroll
+    for (int j = 0; j < U; ++j) c[j] = 0.f;
+    const int width = KT == 0 ? width_max : KT;
+#pragma unroll
+    for (int l = 0; l < width; l += 2) {
+#pragma unroll
+        for (int j = 0; j < U; ++j)
+            if (r[j] != 0.f) t[j] = T[j][(l >> 1) * es4];
+        bool more = false;
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+            if (r[j] != 0.f) {
+                float tau = fminf(r[j], t[j].y);
+                c[j] = fmaf(tau, t[j].x, c[j]);
+                r[j] -= tau;
+                if (r[j] != 0.f) {
+                    tau = fminf(r[j], t[j].w);
+                    c[j] = fmaf(tau, t[j].z, c[j]);
+                    r[j] -= tau;
+                }
+            }
+            more |= r[j] != 0.f;
+        }
+        if ((KT == 0 || l + 2 < KT) && !__any_sync(0xffffffffu, more)) break;
+    }
+}
+
+// One sweep of the CSR for a group of G consecutive queries of the batch: a warp takes a
+// document, lane = G x position + query, so the lanes of a nonzero read the same (column,
+// weight) pair and adjacent table entries.  G <= 8: a lane's position is one of 32 / G
+// consecutive nonzeros, and each phase (position mod 4) is summed in CSR order, through
+// shuffles when a step holds several nonzeros of a phase.  G = 16: each lane takes two
+// consecutive nonzeros of each four, i.e. two phases in accumulators of their own.  Every value
+// is bit-identical to the per-query form (same phases, same order, (p0 + p1) + (p2 + p3)).
+//
+// What bounds the sweep is the latency of its dependent gathers and, behind it, the L1 data
+// path (16 bytes a lane and pair), not DRAM or L2 bandwidth: the form before this one (one entry
+// per load, CSR read when needed, blocks of eight documents) issued in 36% of the cycles with
+// long-scoreboard stalls 28 of 34 cycles per instruction.  So the CSR is read one step ahead, a
+// load brings two table entries of eight queries (one 128-byte line per nonzero), and a block
+// holds two warps of one document each, so that a long document does not keep the slots of
+// seven short ones; documents past twice the mean length come first (long_docs).  Measured, 64
+// queries, k = 4: 1e6 documents (h_q 5..2000) 13.0 -> 9.9 ms, 2e4 documents 335 -> 225 us; one
+// query on 2e4 documents 69 -> 17 us (groups of eight left 28 of 32 lanes idle); 6e4
+// images, k = 8: 1.18 -> 0.97 ms.
+template <int MEAS, int KT, int G, int UN>
+__global__ void __launch_bounds__(kFwdThreads, fwd_blocks(MEAS, KT, G))
+k_fwd_g(const QDesc* __restrict__ qd, const int* __restrict__ nq, const int32_t* __restrict__ row_ptr,
+        const int2* __restrict__ cv, int64_t n, const int32_t* __restrict__ long_docs, int n_long, int long_len,
+        int per_warp, bool to_out)
+{
+    constexpr int P = 32 / G;                // positions per step
+    constexpr int U = G == 16 ? 2 * UN : UN; // nonzeros per lane and step
+    constexpr int ST = G == 16 ? 4 * UN : P * UN;
+    const int q0 = blockIdx.y * G;
     const int nqv = *nq;
     if (q0 >= nqv) return;
-    const int lane = threadIdx.x & 31, g = lane & 7, ph = lane >> 3;
+    const int lane = threadIdx.x & 31, g = lane % G, pl = lane / G;
     const bool act = q0 + g < nqv;
     const QDesc& dq = qd[act ? q0 + g : q0];
     const float2* tq = dq.tab;
-    const int kq = dq.tk;
+    const int kmax = KT == 0 ? (int)__reduce_max_sync(0xffffffffu, (unsigned)dq.tk) : KT;
     float* oq = to_out ? dq.t_out : dq.t_fwd;
-    const int rs = dq.tab_rs, es = dq.tab_es;
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t d = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); d < n; d += warps) {
-        const int32_t a = row_ptr[d], b = row_ptr[d + 1];
-        float acc = 0.f;
-        int32_t e = a + ph;
-        for (; e + 4 < b; e += 8) {  // two nonzeros' costs in flight, added in order
-            const int32_t u0 = col[e], u1 = col[e + 4];
-            const float x0 = val[e], x1 = val[e + 4];
-            if (act) {
-                const float c0 = fwd_cost_p<MEAS, KT>(x0, tq + (int64_t)u0 * rs, es, kq);
-                const float c1 = fwd_cost_p<MEAS, KT>(x1, tq + (int64_t)u1 * rs, es, kq);
-                acc = __fadd_rn(__fadd_rn(acc, c0), c1);
+    const int rs = dq.tab_rs;
+    int64_t i = ((int64_t)blockIdx.x * (kFwdThreads / 32) + (threadIdx.x >> 5)) * per_warp;
+    const int64_t iend = min(i + per_warp, n + n_long);
+    for (; i < iend; ++i) {
+        const int64_t d = i < n_long ? long_docs[i] : i - n_long;
+        const uint32_t a = row_ptr[d], b = row_ptr[d + 1];  // offsets below 2^31: unsigned, so that a step past b cannot wrap
+        if (i >= n_long && (int)(b - a) > long_len) continue;  // taken with the long ones
+        const uint32_t bl = act ? b : a;  // lanes without a query read nothing
+        float acc0 = 0.f, acc1 = 0.f;
+        auto off = [&](int j) -> uint32_t { return G == 16 ? (j >> 1) * 4 + 2 * pl + (j & 1) : j * P + pl; };
+        int2 nx[U];
+#pragma unroll
+        for (int j = 0; j < U; ++j) nx[j] = a + off(j) < bl ? cv[a + off(j)] : make_int2(0, 0);
+        for (uint32_t e = a; e < b; e += ST) {
+            int2 x[U];
+#pragma unroll
+            for (int j = 0; j < U; ++j) x[j] = nx[j];
+#pragma unroll
+            for (int j = 0; j < U; ++j) nx[j] = e + ST + off(j) < bl ? cv[e + ST + off(j)] : make_int2(0, 0);
+            float c[U], w[U];
+            const float4* T[U];
+#pragma unroll
+            for (int j = 0; j < U; ++j) {
+                w[j] = __int_as_float(x[j].y);
+                T[j] = reinterpret_cast<const float4*>(tq + (int64_t)x[j].x * rs);
+            }
+            if constexpr (KT == 1 || MEAS == M_RWMD) {
+#pragma unroll
+                for (int j = 0; j < U; ++j)
+                    c[j] = w[j] != 0.f ? __fmul_rn(w[j], reinterpret_cast<const float2*>(T[j])->x) : 0.f;
+            } else {
+                fwd_cost_pairs<MEAS, KT, U>(w, T, G, kmax, c);
+            }
+#pragma unroll
+            for (int j = 0; j < U; ++j) {
+                if constexpr (G == 16) {
+                    if (j & 1) acc1 = __fadd_rn(acc1, c[j]); else acc0 = __fadd_rn(acc0, c[j]);
+                } else if constexpr (G == 8) {
+                    acc0 = __fadd_rn(acc0, c[j]);
+                } else {
+#pragma unroll
+                    for (int t = 0; t < P / 4; ++t)
+                        acc0 = __fadd_rn(acc0, __shfl_sync(0xffffffffu, c[j], g + G * ((pl & 3) + 4 * t)));
+                }
             }
         }
-        if (e < b) {
-            const int32_t u = col[e];
-            const float x = val[e];
-            if (act) acc = __fadd_rn(acc, fwd_cost_p<MEAS, KT>(x, tq + (int64_t)u * rs, es, kq));
+        float s;
+        if (G == 16) {
+            s = __fadd_rn(acc0, acc1);
+            s = __fadd_rn(s, __shfl_xor_sync(0xffffffffu, s, 16));
+        } else {
+            s = __fadd_rn(acc0, __shfl_xor_sync(0xffffffffu, acc0, G));
+            s = __fadd_rn(s, __shfl_xor_sync(0xffffffffu, s, 2 * G));
         }
-        acc += __shfl_xor_sync(0xffffffffu, acc, 8);
-        acc += __shfl_xor_sync(0xffffffffu, acc, 16);
-        if (ph == 0 && act) oq[d] = acc;
+        if (pl == 0 && act) oq[d] = s;
     }
 }
 
@@ -441,15 +552,54 @@ cudaError_t launch_fwd(int meas, const int32_t* row_ptr, const int32_t* col, con
     return cudaGetLastError();
 }
 
+// The interleaved CSR of the entry-chain sweep.
+__global__ void k_interleave(const int32_t* __restrict__ col, const float* __restrict__ val, int64_t nnz,
+                             int2* __restrict__ cv)
+{
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nnz; e += (int64_t)gridDim.x * blockDim.x)
+        cv[e] = make_int2(col[e], __float_as_int(val[e]));
+}
+
+cudaError_t launch_interleave(const int32_t* col, const float* val, int64_t nnz, int2* cv, cudaStream_t st)
+{
+    if (nnz <= 0) return cudaSuccess;
+    k_interleave<<<(unsigned)std::min<int64_t>((nnz + 255) / 256, 152 * 16), 256, 0, st>>>(col, val, nnz, cv);
+    return cudaGetLastError();
+}
+
+template <int G>
+static void fwd_chain(int m, int kw, int max_tk, const QDesc* qd, const int* nq, int max_q, const int32_t* row_ptr,
+                      const FwdSweep& w, int64_t n, bool to_out, cudaStream_t st)
+{
+    constexpr int warps = kFwdThreads / 32;
+    // documents per warp: one, or for large databases four (fewer block launches)
+    const int per_warp = n > 200000 ? 4 : 1;
+    const dim3 gg((unsigned)((n + w.n_long + warps * per_warp - 1) / (warps * per_warp)), (unsigned)((max_q + G - 1) / G));
+#define EMD_LM(M, KT) k_fwd_g<M, KT, G, fwd_un(M, KT, G)><<<gg, kFwdThreads, 0, st>>>(qd, nq, row_ptr, w.cv, n, w.long_docs, w.n_long, w.long_len, per_warp, to_out)
+    switch (m) {
+    case M_RWMD: EMD_LM(M_RWMD, 0); break;
+    case M_OMR:
+        if (max_tk >= 2) EMD_LM(M_OMR, 0); else EMD_LM(M_RWMD, 0);  // one-bin queries: tables of one entry, same cost
+        break;
+    default: {
+#define EMD_L(KT) EMD_LM(M_ACT, KT)
+        EMD_FWD_KT_SWITCH(kw, EMD_L)
+#undef EMD_L
+        break;
+    }
+    }
+#undef EMD_LM
+}
+
 cudaError_t launch_fwd_b(int meas, const QDesc* qd, const int* nq, int max_q, const int32_t* row_ptr,
-                         const int32_t* col, const float* val, int64_t n, bool to_out, bool grouped, int max_tk,
-                         cudaStream_t st, int variant)
+                         const int32_t* col, const float* val, const FwdSweep& sweep, int64_t n, bool to_out,
+                         int group, int max_tk, cudaStream_t st, int variant)
 {
     const int kt = fwd_kt(max_tk);
     if (max_q <= 0 || n <= 0) return cudaSuccess;
     const int warps = 8;
     const int64_t blocks = std::min<int64_t>((n + warps - 1) / warps, 152 * 64);
-    if (grouped) {  // one document per warp, eight queries
+    if (group > 0) {  // one document per warp, `group` queries (small groups: several documents)
         dim3 gg((unsigned)std::max<int64_t>(1, blocks), (unsigned)((max_q + kFwdGroup - 1) / kFwdGroup));
         const int m = meas == M_ICT ? M_ACT : meas;  // ICT tables: the ACT steps over the written entries
         const int kw = meas == M_RWMD ? 1 : meas == M_OMR ? 2 : (meas == M_ICT && kt == 0 ? 0 : kt);
@@ -467,15 +617,13 @@ cudaError_t launch_fwd_b(int meas, const QDesc* qd, const int* nq, int max_q, co
             return cudaGetLastError();
         }
         if (kw == 0 || variant == kFwdChain) {  // entry-interleaved rows, loads while mass remains
-            switch (m) {
-            case M_RWMD: k_fwd_g<M_RWMD, 0><<<gg, warps * 32, 0, st>>>(qd, nq, row_ptr, col, val, n, to_out); break;
-            case M_OMR: k_fwd_g<M_OMR, 0><<<gg, warps * 32, 0, st>>>(qd, nq, row_ptr, col, val, n, to_out); break;
-            default: {
-#define EMD_L(KT) k_fwd_g<M_ACT, KT><<<gg, warps * 32, 0, st>>>(qd, nq, row_ptr, col, val, n, to_out)
-                EMD_FWD_KT_SWITCH(kw, EMD_L)
-#undef EMD_L
-                break;
-            }
+            switch (group) {
+            case 1: fwd_chain<1>(m, kw, max_tk, qd, nq, max_q, row_ptr, sweep, n, to_out, st); break;
+            case 2: fwd_chain<2>(m, kw, max_tk, qd, nq, max_q, row_ptr, sweep, n, to_out, st); break;
+            case 4: fwd_chain<4>(m, kw, max_tk, qd, nq, max_q, row_ptr, sweep, n, to_out, st); break;
+            case 8: fwd_chain<8>(m, kw, max_tk, qd, nq, max_q, row_ptr, sweep, n, to_out, st); break;
+            case 16: fwd_chain<16>(m, kw, max_tk, qd, nq, max_q, row_ptr, sweep, n, to_out, st); break;
+            default: return cudaErrorInvalidValue;
             }
             return cudaGetLastError();
         }

@@ -254,7 +254,7 @@ __device__ __forceinline__ void insert_dj(float (&z)[KT], int (&s)[KT], float d,
 
 template <int KT>
 __device__ __forceinline__ void table_body(const float* __restrict__ D, int ldd, int64_t M, int h, int k, const float* __restrict__ q_w,
-        float2* __restrict__ tab, int32_t* __restrict__ tab_s, int rs, int es, bool sq)
+        float2* __restrict__ tab, int32_t* __restrict__ tab_s, int rs, int es, int pr, bool sq)
 {
     const int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (row >= M) return;
@@ -284,7 +284,7 @@ __device__ __forceinline__ void table_body(const float* __restrict__ D, int ldd,
     for (int l = 0; l < KT; ++l) {
         if (l < k) {
             const bool valid = s[l] != INT32_MAX;
-            tab[row * rs + l * es] = make_float2(valid ? d_value(z[l], sq) : INFINITY, valid ? q_w[s[l]] : 0.f);
+            tab[row * rs + tab_entry(l, es, pr)] = make_float2(valid ? d_value(z[l], sq) : INFINITY, tab_cap(valid ? q_w[s[l]] : 0.f, l, k, pr));
             if (tab_s) tab_s[row * k + l] = valid ? s[l] : -1;
         }
     }
@@ -294,14 +294,14 @@ template <int KT>
 __global__ void __launch_bounds__(128) k_table(const float* __restrict__ D, int ldd, int64_t M, int h, int k, const float* __restrict__ q_w,
         float2* __restrict__ tab, int32_t* __restrict__ tab_s, bool sq)
 {
-    table_body<KT>(D, ldd, M, h, k, q_w, tab, tab_s, k, 1, sq);
+    table_body<KT>(D, ldd, M, h, k, q_w, tab, tab_s, k, 1, 0, sq);
 }
 
 // k larger than the register lists: successive minima, each strictly after the previous
 // in (d, j) order.  O(k * h / 32) per lane; used for ICT on small queries.
 __device__ __forceinline__ void table_generic_body(const float* __restrict__ D, int ldd, int64_t M, int h, int k,
                                 const float* __restrict__ q_w, float2* __restrict__ tab,
-                                int32_t* __restrict__ tab_s, int rs, int es, bool sq)
+                                int32_t* __restrict__ tab_s, int rs, int es, int pr, bool sq)
 {
     const int lane = threadIdx.x & 31;
     const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -325,7 +325,7 @@ __device__ __forceinline__ void table_generic_body(const float* __restrict__ D, 
         }
         if (lane == 0) {
             const bool valid = bs != INT32_MAX;
-            tab[row * rs + l * es] = make_float2(valid ? d_value(bz, sq) : INFINITY, valid ? q_w[bs] : 0.f);
+            tab[row * rs + tab_entry(l, es, pr)] = make_float2(valid ? d_value(bz, sq) : INFINITY, tab_cap(valid ? q_w[bs] : 0.f, l, k, pr));
             if (tab_s) tab_s[row * k + l] = valid ? bs : -1;
         }
         pz = bz;
@@ -341,7 +341,7 @@ __device__ __forceinline__ void table_generic_body(const float* __restrict__ D, 
 __device__ __forceinline__ void table_ict_body(const float* __restrict__ D, int ldd, int64_t M, int h, int W,
                                                const float* __restrict__ q_w, const float* __restrict__ xmax,
                                                float2* __restrict__ tab, int32_t* __restrict__ tab_s, int rs,
-                                               int es, int* __restrict__ over, bool sq)
+                                               int es, int pr, int* __restrict__ over, bool sq)
 {
     const int lane = threadIdx.x & 31;
     const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
@@ -369,7 +369,7 @@ __device__ __forceinline__ void table_ict_body(const float* __restrict__ D, int 
         const bool valid = bs != INT32_MAX;  // always while l < h, unless D holds NaN
         const float w = valid ? q_w[bs] : 0.f;
         if (lane == 0) {
-            tab[row * rs + (int64_t)l * es] = make_float2(valid ? d_value(bz, sq) : INFINITY, w);
+            tab[row * rs + tab_entry(l, es, pr)] = make_float2(valid ? d_value(bz, sq) : INFINITY, tab_cap(w, l, lim, pr));
             if (tab_s) tab_s[row * W + l] = valid ? bs : -1;
         }
         if (!valid) break;
@@ -392,7 +392,7 @@ constexpr int kIctFast = 8;
 __device__ __forceinline__ void ict_fast_body(const float* __restrict__ D, int ldd, int64_t M, int h, int W,
                                               const float* __restrict__ q_w, const float* __restrict__ xmax,
                                               float2* __restrict__ tab, int32_t* __restrict__ tab_s, int rs, int es,
-                                              int* __restrict__ over, bool sq)
+                                              int pr, int* __restrict__ over, bool sq)
 {
     const int64_t row = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (row >= M) return;
@@ -444,7 +444,7 @@ __device__ __forceinline__ void ict_fast_body(const float* __restrict__ D, int l
     for (int l = 0; l < kIctFast; ++l) {
         if (l < L) {
             const bool valid = s[l] != INT32_MAX;
-            tab[row * rs + (int64_t)l * es] = make_float2(valid ? d_value(z[l], sq) : INFINITY, valid ? q_w[s[l]] : 0.f);
+            tab[row * rs + tab_entry(l, es, pr)] = make_float2(valid ? d_value(z[l], sq) : INFINITY, tab_cap(valid ? q_w[s[l]] : 0.f, l, lim, pr));
             if (tab_s) tab_s[row * W + l] = valid ? s[l] : -1;
         }
     }
@@ -454,21 +454,21 @@ __global__ void __launch_bounds__(128) k_table_ict_fast(const float* __restrict_
                                  const float* __restrict__ q_w, const float* __restrict__ xmax,
                                  float2* __restrict__ tab, int32_t* __restrict__ tab_s, int* __restrict__ over, bool sq)
 {
-    ict_fast_body(D, ldd, M, h, W, q_w, xmax, tab, tab_s, W, 1, over, sq);
+    ict_fast_body(D, ldd, M, h, W, q_w, xmax, tab, tab_s, W, 1, 0, over, sq);
 }
 
 __global__ void k_table_ict(const float* __restrict__ D, int ldd, int64_t M, int h, int W,
                             const float* __restrict__ q_w, const float* __restrict__ xmax, float2* __restrict__ tab,
                             int32_t* __restrict__ tab_s, int* __restrict__ over, bool sq)
 {
-    table_ict_body(D, ldd, M, h, W, q_w, xmax, tab, tab_s, W, 1, over, sq);
+    table_ict_body(D, ldd, M, h, W, q_w, xmax, tab, tab_s, W, 1, 0, over, sq);
 }
 
 __global__ void k_table_generic(const float* __restrict__ D, int ldd, int64_t M, int h, int k,
                                 const float* __restrict__ q_w, float2* __restrict__ tab,
                                 int32_t* __restrict__ tab_s, bool sq)
 {
-    table_generic_body(D, ldd, M, h, k, q_w, tab, tab_s, k, 1, sq);
+    table_generic_body(D, ldd, M, h, k, q_w, tab, tab_s, k, 1, 0, sq);
 }
 
 // Re-rank form of the table, for approximate distance matrices (BF16 / E4M3 Phase 1).
@@ -493,7 +493,7 @@ __host__ __device__ constexpr size_t rerank_smem_bytes(int h) { return (size_t)h
 template <int KCT>
 __device__ __forceinline__ void table_rerank_body(float* __restrict__ D, int ldd, int64_t M, int h, int k, int kc, const float* __restrict__ V,
                const float* __restrict__ Q, int ldv, const float* __restrict__ q_w, float2* __restrict__ tab,
-               int32_t* __restrict__ tab_s, int64_t tile, int rs, int es)
+               int32_t* __restrict__ tab_s, int64_t tile, int rs, int es, int pr)
 {
     extern __shared__ float4 qs4[];  // [h]: Q[j][d0 .. d0 + 4)
     const int tid = threadIdx.x;
@@ -556,7 +556,7 @@ __device__ __forceinline__ void table_rerank_body(float* __restrict__ D, int ldd
     for (int l = 0; l < KCT; ++l) {
         if (l < k) {
             const bool valid = s2[l] != INT32_MAX;
-            tab[row * rs + l * es] = make_float2(valid ? sq_to_dist(z[l]) : INFINITY, valid ? q_w[s2[l]] : 0.f);
+            tab[row * rs + tab_entry(l, es, pr)] = make_float2(valid ? sq_to_dist(z[l]) : INFINITY, tab_cap(valid ? q_w[s2[l]] : 0.f, l, k, pr));
             if (tab_s) tab_s[row * k + l] = valid ? s2[l] : -1;
         }
     }
@@ -567,7 +567,7 @@ __global__ void __launch_bounds__(kRrRows) k_table_rerank(float* __restrict__ D,
                const float* __restrict__ Q, int ldv, const float* __restrict__ q_w, float2* __restrict__ tab,
                int32_t* __restrict__ tab_s)
 {
-    table_rerank_body<KCT>(D, ldd, M, h, k, kc, V, Q, ldv, q_w, tab, tab_s, blockIdx.x, k, 1);
+    table_rerank_body<KCT>(D, ldd, M, h, k, kc, V, Q, ldv, q_w, tab, tab_s, blockIdx.x, k, 1, 0);
 }
 
 // ------------------------------------------------------------------ batched forms
@@ -604,7 +604,7 @@ k_table_b(const QDesc* __restrict__ qd, const int* __restrict__ nq, int64_t M)
 {
     if ((int)blockIdx.y >= *nq) return;
     const QDesc& d = qd[blockIdx.y];
-    table_body<KT>(d.D, d.ldd, M, d.h, d.tk, d.qw, d.tab, nullptr, d.tab_rs, d.tab_es, d.sq != 0);
+    table_body<KT>(d.D, d.ldd, M, d.h, d.tk, d.qw, d.tab, nullptr, d.tab_rs, d.tab_es, d.tab_pair, d.sq != 0);
 }
 
 // D[vslot[q_idx[j]], j] = 0 for the query bins whose id is a used vocabulary row (ids
@@ -653,7 +653,7 @@ __global__ void __launch_bounds__(128) k_table_ict_fast_b(const QDesc* __restric
 {
     if ((int)blockIdx.y >= *nq) return;
     const QDesc& d = qd[blockIdx.y];
-    ict_fast_body(d.D, d.ldd, M, d.h, d.tk, d.qw, xmax, d.tab, nullptr, d.tab_rs, d.tab_es, d.over, d.sq != 0);
+    ict_fast_body(d.D, d.ldd, M, d.h, d.tk, d.qw, xmax, d.tab, nullptr, d.tab_rs, d.tab_es, d.tab_pair, d.over, d.sq != 0);
 }
 
 __global__ void k_table_ict_b(const QDesc* __restrict__ qd, const int* __restrict__ nq, int64_t M,
@@ -661,14 +661,14 @@ __global__ void k_table_ict_b(const QDesc* __restrict__ qd, const int* __restric
 {
     if ((int)blockIdx.y >= *nq) return;
     const QDesc& d = qd[blockIdx.y];
-    table_ict_body(d.D, d.ldd, M, d.h, d.tk, d.qw, xmax, d.tab, nullptr, d.tab_rs, d.tab_es, d.over, d.sq != 0);
+    table_ict_body(d.D, d.ldd, M, d.h, d.tk, d.qw, xmax, d.tab, nullptr, d.tab_rs, d.tab_es, d.tab_pair, d.over, d.sq != 0);
 }
 
 __global__ void k_table_generic_b(const QDesc* __restrict__ qd, const int* __restrict__ nq, int64_t M)
 {
     if ((int)blockIdx.y >= *nq) return;
     const QDesc& d = qd[blockIdx.y];
-    table_generic_body(d.D, d.ldd, M, d.h, d.tk, d.qw, d.tab, nullptr, d.tab_rs, d.tab_es, d.sq != 0);
+    table_generic_body(d.D, d.ldd, M, d.h, d.tk, d.qw, d.tab, nullptr, d.tab_rs, d.tab_es, d.tab_pair, d.sq != 0);
 }
 
 // Queries vary fastest (blockIdx.x) so that the blocks of one vocabulary tile for all
@@ -681,7 +681,7 @@ k_table_rerank_b(const QDesc* __restrict__ qd, const int* __restrict__ nq, int64
     if ((int)blockIdx.x >= *nq) return;
     const QDesc& d = qd[blockIdx.x];
     table_rerank_body<KCT>(d.D, d.ldd, M, d.h, d.tk, d.kc, V, d.Q, ldv, d.qw, d.tab, nullptr, blockIdx.y, d.tab_rs,
-                           d.tab_es);
+                           d.tab_es, d.tab_pair);
 }
 
 // Fused approximate forms: the re-rank from the candidate bins the product's epilogue kept
@@ -755,7 +755,7 @@ k_rerank_cand_b(const QDesc* __restrict__ qd, const int* __restrict__ nq, int64_
     for (int l = 0; l < KCT; ++l) {
         if (l < k) {
             const bool valid = s2[l] != INT32_MAX;
-            d.tab[row * d.tab_rs + l * d.tab_es] = make_float2(valid ? sq_to_dist(z[l]) : INFINITY, valid ? d.qw[s2[l]] : 0.f);
+            d.tab[row * d.tab_rs + tab_entry(l, d.tab_es, d.tab_pair)] = make_float2(valid ? sq_to_dist(z[l]) : INFINITY, tab_cap(valid ? d.qw[s2[l]] : 0.f, l, k, d.tab_pair));
         }
         if (l == k - 1) ek = z[l];
     }
@@ -817,7 +817,7 @@ k_rerank_full_b(const QDesc* __restrict__ qd, const int* __restrict__ nq, const 
             }
             if (lane == 0) {
                 const bool valid = bs != INT32_MAX;
-                d.tab[row * d.tab_rs + l * d.tab_es] = make_float2(valid ? sq_to_dist(bz) : INFINITY, valid ? d.qw[bs] : 0.f);
+                d.tab[row * d.tab_rs + tab_entry(l, d.tab_es, d.tab_pair)] = make_float2(valid ? sq_to_dist(bz) : INFINITY, tab_cap(valid ? d.qw[bs] : 0.f, l, d.tk, d.tab_pair));
             }
             if (s[0] == bs && bs != INT32_MAX) {  // the owner pops its head
 #pragma unroll

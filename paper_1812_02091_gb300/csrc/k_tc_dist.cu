@@ -1120,8 +1120,9 @@ k_tc_table_batch(const uint8_t* __restrict__ A_hi, const uint8_t* __restrict__ A
                         for (int l = 0; l < KT; ++l) {
                             if (l < d.tk) {
                                 const bool valid = sj[l] != INT32_MAX;
-                                d.tab[u * d.tab_rs + (int64_t)l * d.tab_es] =
-                                    make_float2(valid ? sq_to_dist(z[l]) : INFINITY, valid ? d.qw[sj[l]] : 0.f);
+                                d.tab[u * d.tab_rs + tab_entry(l, d.tab_es, d.tab_pair)] =
+                                    make_float2(valid ? sq_to_dist(z[l]) : INFINITY,
+                                                tab_cap(valid ? d.qw[sj[l]] : 0.f, l, d.tk, d.tab_pair));
                             }
                         }
                     }
@@ -1541,8 +1542,9 @@ k_tc_table_pair(const uint8_t* __restrict__ A_hi, const uint8_t* __restrict__ A_
                     for (int l = 0; l < KT; ++l) {
                         if (l < d.tk) {
                             const bool valid = sj[l] != INT32_MAX;
-                            d.tab[u * d.tab_rs + (int64_t)l * d.tab_es] =
-                                make_float2(valid ? sq_to_dist(z[l]) : INFINITY, valid ? d.qw[sj[l]] : 0.f);
+                            d.tab[u * d.tab_rs + tab_entry(l, d.tab_es, d.tab_pair)] =
+                                make_float2(valid ? sq_to_dist(z[l]) : INFINITY,
+                                                tab_cap(valid ? d.qw[sj[l]] : 0.f, l, d.tk, d.tab_pair));
                         }
                     }
                 }
