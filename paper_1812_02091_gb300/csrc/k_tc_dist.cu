@@ -102,6 +102,13 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint64
     return true;
 }
 
+// The same with the time limit counted from the first failed try: a wait that is already over
+// reads no clock.
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity)
+{
+    return mbar_try_wait(bar, parity) || mbar_wait(bar, parity, global_ns() + TC_TIMEOUT_NS);
+}
+
 __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar)
 {
     asm volatile(
@@ -220,6 +227,23 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar)
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
+// One K step of a split product (or of a single-part one): hi times [hi | lo] as one product of
+// 2 Nt columns -- the query chunk's lo rows follow its hi rows in shared memory and the cross
+// terms' accumulator follows the main one in TMEM -- then lo times hi onto the cross terms.  The
+// vocabulary rows are read twice instead of three times from shared memory, whose bandwidth the
+// 128-column products exceed (fused table, 64 text queries: 2.10 -> 1.93 ms).
+template <int FMT>
+__device__ __forceinline__ void mma_step(uint32_t acc0, int Nt, uint64_t da, uint64_t da_lo, uint64_t db, uint32_t idesc,
+                                         uint32_t accumulate)
+{
+    if (FMT == TC_SPLIT) {
+        mma_issue<FMT>(acc0, da, db, idesc + ((uint32_t)(Nt >> 3) << 17), accumulate);
+        mma_issue<FMT>(acc0 + (uint32_t)Nt, da_lo, db, idesc, 1u);
+    } else {
+        mma_issue<FMT>(acc0, da, db, idesc, accumulate);
+    }
+}
+
 // Persistent form: each CTA (one per SM) walks tiles t = blockIdx.x, += gridDim.x in
 // column-tile-major order (t -> column tile t / m_tiles, row tile t % m_tiles), so a CTA's
 // consecutive tiles nearly always share their query columns.  The query panel (all K
@@ -297,7 +321,7 @@ k_tc_dist(const uint8_t* __restrict__ A_hi, const uint8_t* __restrict__ A_lo, in
             const int64_t m0 = (int64_t)(t % m_tiles) * TC_BM;
             const int nt = t / m_tiles;
             if (nt != cur_n) {
-                if (reloads > 0 && !mbar_wait(bfree, (uint32_t)(reloads - 1) & 1u, global_ns() + TC_TIMEOUT_NS)) {
+                if (reloads > 0 && !mbar_wait(bfree, (uint32_t)(reloads - 1) & 1u)) {
                     fail();
                     break;
                 }
@@ -315,7 +339,7 @@ k_tc_dist(const uint8_t* __restrict__ A_hi, const uint8_t* __restrict__ A_lo, in
             }
             for (int c = 0; c < KC; ++c, ++g) {
                 const int s = (int)(g % stages);
-                if (g >= stages && !mbar_wait(&empty[s], (uint32_t)((g / stages) - 1) & 1u, global_ns() + TC_TIMEOUT_NS)) {
+                if (g >= stages && !mbar_wait(&empty[s], (uint32_t)((g / stages) - 1) & 1u)) {
                     fail();
                     break;
                 }
@@ -343,7 +367,7 @@ k_tc_dist(const uint8_t* __restrict__ A_hi, const uint8_t* __restrict__ A_lo, in
                                    ((uint32_t)(Nt >> 3) << 17) | ((uint32_t)(TC_BM >> 4) << 24);
             if (nt != cur_n) {
                 if (reloads > 0) mma_commit(bfree);  // the old panel is released once its MMAs finish
-                if (!mbar_wait(bfull, (uint32_t)reloads & 1u, global_ns() + TC_TIMEOUT_NS)) {
+                if (!mbar_wait(bfull, (uint32_t)reloads & 1u)) {
                     fail();
                     break;
                 }
@@ -351,7 +375,7 @@ k_tc_dist(const uint8_t* __restrict__ A_hi, const uint8_t* __restrict__ A_lo, in
                 ++reloads;
             }
             const int buf = it & 1;
-            if (it >= 2 && !mbar_wait(&tempty[buf], (uint32_t)((it >> 1) - 1) & 1u, global_ns() + TC_TIMEOUT_NS)) {
+            if (it >= 2 && !mbar_wait(&tempty[buf], (uint32_t)((it >> 1) - 1) & 1u)) {
                 fail();
                 break;
             }
@@ -360,7 +384,7 @@ k_tc_dist(const uint8_t* __restrict__ A_hi, const uint8_t* __restrict__ A_lo, in
             bool ok = true;
             for (int c = 0; c < KC; ++c, ++g) {
                 const int s = (int)(g % stages);
-                if (!mbar_wait(&full[s], (uint32_t)(g / stages) & 1u, global_ns() + TC_TIMEOUT_NS)) {
+                if (!mbar_wait(&full[s], (uint32_t)(g / stages) & 1u)) {
                     fail();
                     ok = false;
                     break;
@@ -402,7 +426,7 @@ k_tc_dist(const uint8_t* __restrict__ A_hi, const uint8_t* __restrict__ A_lo, in
             const int n0 = (t / m_tiles) * TC_BN;
             const int Nt = min(TC_BN, (int)round_up(N - n0, 16));
             const int buf = it & 1;
-            if (!mbar_wait(&tfull[buf], (uint32_t)(it >> 1) & 1u, global_ns() + TC_TIMEOUT_NS)) {
+            if (!mbar_wait(&tfull[buf], (uint32_t)(it >> 1) & 1u)) {
                 fail();
                 break;
             }
@@ -535,7 +559,7 @@ k_tc_dist_batch(const uint8_t* __restrict__ A_hi, const uint8_t* __restrict__ A_
         bool ok = true;
         for (int w = blockIdx.x; w < total && ok && !*abort_flag; w += gridDim.x, ++items) {
             const int64_t m0 = (int64_t)(w % m_tiles) * TC_BM;
-            if (items > 0 && !mbar_wait(afree, (uint32_t)(items - 1) & 1u, global_ns() + TC_TIMEOUT_NS)) {
+            if (items > 0 && !mbar_wait(afree, (uint32_t)(items - 1) & 1u)) {
                 fail();
                 break;
             }
@@ -557,7 +581,7 @@ k_tc_dist_batch(const uint8_t* __restrict__ A_hi, const uint8_t* __restrict__ A_
                     for (int c = 0; c < KC; ++c, ++gb, rs = rs + 1 == stages ? (rp ^= 1u, 0) : rs + 1) {
                         const int s = rs;
                         if (gb >= stages &&
-                            !mbar_wait(&empty[s], rp ^ 1u, global_ns() + TC_TIMEOUT_NS)) {
+                            !mbar_wait(&empty[s], rp ^ 1u)) {
                             fail();
                             ok = false;
                             break;
@@ -565,7 +589,7 @@ k_tc_dist_batch(const uint8_t* __restrict__ A_hi, const uint8_t* __restrict__ A_
                         uint8_t* bst = bring + (size_t)s * kBStage;
                         mbar_expect_tx(&full[s], (uint32_t)kParts * b_bytes);
                         bulk_g2s(bst, bh + ((int64_t)c * d.npad + n0) * EB, b_bytes, &full[s]);
-                        if (SPLIT) bulk_g2s(bst + kBBytes, bl + ((int64_t)c * d.npad + n0) * EB, b_bytes, &full[s]);
+                        if (SPLIT) bulk_g2s(bst + b_bytes, bl + ((int64_t)c * d.npad + n0) * EB, b_bytes, &full[s]);
                     }
                 }
             }
@@ -582,7 +606,7 @@ k_tc_dist_batch(const uint8_t* __restrict__ A_hi, const uint8_t* __restrict__ A_
         int it = 0, items = 0;
         bool ok = true;
         for (int w = blockIdx.x; w < total && ok && !*abort_flag; w += gridDim.x, ++items) {
-            if (!mbar_wait(afull, (uint32_t)items & 1u, global_ns() + TC_TIMEOUT_NS)) {
+            if (!mbar_wait(afull, (uint32_t)items & 1u)) {
                 fail();
                 break;
             }
@@ -595,7 +619,7 @@ k_tc_dist_batch(const uint8_t* __restrict__ A_hi, const uint8_t* __restrict__ A_
                     const uint32_t idesc = (1u << 4) | (TcFmt<FMT>::atype << 7) | (TcFmt<FMT>::atype << 10) |
                                            ((uint32_t)(Nt >> 3) << 17) | ((uint32_t)(TC_BM >> 4) << 24);
                     const int buf = it & 1;
-                    if (it >= 2 && !mbar_wait(&tempty[buf], (uint32_t)((it >> 1) - 1) & 1u, global_ns() + TC_TIMEOUT_NS)) {
+                    if (it >= 2 && !mbar_wait(&tempty[buf], (uint32_t)((it >> 1) - 1) & 1u)) {
                         fail();
                         ok = false;
                         break;
@@ -604,7 +628,7 @@ k_tc_dist_batch(const uint8_t* __restrict__ A_hi, const uint8_t* __restrict__ A_
                     const uint32_t acc0 = tmem + (uint32_t)buf * kAcc;
                     for (int c = 0; c < KC; ++c, ++gb, rs = rs + 1 == stages ? (rp ^= 1u, 0) : rs + 1) {
                         const int s = rs;
-                        if (!mbar_wait(&full[s], rp, global_ns() + TC_TIMEOUT_NS)) {
+                        if (!mbar_wait(&full[s], rp)) {
                             fail();
                             ok = false;
                             break;
@@ -613,11 +637,10 @@ k_tc_dist_batch(const uint8_t* __restrict__ A_hi, const uint8_t* __restrict__ A_
                         const uint32_t sa = smem_u32(apanel + (size_t)c * kAChunk);
                         const uint32_t sa_lo = sa + kABytes;
                         const uint32_t sb = smem_u32(bring + (size_t)s * kBStage);
-                        const uint32_t sb_lo = sb + kBBytes;
                         // descriptors of the chunk's first K step; a step of 16 elements (256 B) adds 16 to the
                         // address field (addresses stay below 2^18, so no carry leaves the 14-bit field)
                         const uint64_t dA0 = smem_desc(sa, kSbo), dB0 = smem_desc(sb, kSbo);
-                        const uint64_t dAl0 = smem_desc(sa_lo, kSbo), dBl0 = smem_desc(sb_lo, kSbo);
+                        const uint64_t dAl0 = smem_desc(sa_lo, kSbo);
 #pragma unroll
                         for (int ks = 0; ks < (int)TcFmt<FMT>::mmas; ++ks) {
                             if (c == KC - 1 && ks >= klast) break;  // the last chunk's zero K steps
@@ -625,11 +648,7 @@ k_tc_dist_batch(const uint8_t* __restrict__ A_hi, const uint8_t* __restrict__ A_
                             const uint32_t acc = (c > 0 || ks > 0) ? 1u : 0u;
                             const uint64_t kd = (uint64_t)(ko >> 4);
                             const uint64_t da = dA0 + kd, db = dB0 + kd;
-                            mma_issue<FMT>(acc0, da, db, idesc, acc);
-                            if (SPLIT) {
-                                mma_issue<FMT>(acc0 + 128, da, dBl0 + kd, idesc, acc);
-                                mma_issue<FMT>(acc0 + 128, dAl0 + kd, db, idesc, 1u);
-                            }
+                            mma_step<FMT>(acc0, Nt, da, dAl0 + kd, db, idesc, acc);
                         }
                         mma_commit(&empty[s]);
                     }
@@ -668,7 +687,7 @@ k_tc_dist_batch(const uint8_t* __restrict__ A_hi, const uint8_t* __restrict__ A_
                     const bool lok = lcol < N;
                     const float cb_l = lok ? -2.f * qsc[lcol] : 0.f;
                     const float nb_l = lok ? qnm[lcol] : 0.f;
-                    if (!mbar_wait(&tfull[buf], (uint32_t)(it >> 1) & 1u, global_ns() + TC_TIMEOUT_NS)) {
+                    if (!mbar_wait(&tfull[buf], (uint32_t)(it >> 1) & 1u)) {
                         fail();
                         ok = false;
                         break;
@@ -682,7 +701,7 @@ k_tc_dist_batch(const uint8_t* __restrict__ A_hi, const uint8_t* __restrict__ A_
                         for (int hh = 0; hh < 2; ++hh) {  // two halves of 16 columns
                         uint32_t r0[16], r1[16];
                         tmem_ld16(tbase + (uint32_t)(cc + 16 * hh), r0);
-                        if (SPLIT) tmem_ld16(tbase + 128u + (uint32_t)(cc + 16 * hh), r1);
+                        if (SPLIT) tmem_ld16(tbase + (uint32_t)Nt + (uint32_t)(cc + 16 * hh), r1);
                         tmem_wait_ld();
 #pragma unroll
                         for (int e4 = 4 * hh; e4 < 4 * hh + 4; ++e4) {
@@ -889,7 +908,7 @@ k_tc_table_batch(const uint8_t* __restrict__ A_hi, const uint8_t* __restrict__ A
         bool ok = true;
         for (int w = blockIdx.x; w < total && ok && !*abort_flag; w += gridDim.x, ++items) {
             const int64_t m0 = (int64_t)(w % m_tiles) * TC_BM;
-            if (items > 0 && !mbar_wait(afree, (uint32_t)(items - 1) & 1u, global_ns() + TC_TIMEOUT_NS)) {
+            if (items > 0 && !mbar_wait(afree, (uint32_t)(items - 1) & 1u)) {
                 fail();
                 break;
             }
@@ -912,7 +931,7 @@ k_tc_table_batch(const uint8_t* __restrict__ A_hi, const uint8_t* __restrict__ A
                 for (int c = 0; c < KC; ++c, ++gb, rs = rs + 1 == stages ? (rp ^= 1u, 0) : rs + 1) {
                     const int st = rs;
                     if (gb >= stages &&
-                        !mbar_wait(&empty[st], rp ^ 1u, global_ns() + TC_TIMEOUT_NS)) {
+                        !mbar_wait(&empty[st], rp ^ 1u)) {
                         fail();
                         ok = false;
                         break;
@@ -920,7 +939,7 @@ k_tc_table_batch(const uint8_t* __restrict__ A_hi, const uint8_t* __restrict__ A
                     uint8_t* bst = bring + (size_t)st * kBStage;
                     mbar_expect_tx(&full[st], (uint32_t)kParts * b_bytes);
                     bulk_g2s(bst, bh + ((int64_t)c * d.npad + n0) * EB, b_bytes, &full[st]);
-                    if (SPLIT) bulk_g2s(bst + kBBytes, bl + ((int64_t)c * d.npad + n0) * EB, b_bytes, &full[st]);
+                    if (SPLIT) bulk_g2s(bst + b_bytes, bl + ((int64_t)c * d.npad + n0) * EB, b_bytes, &full[st]);
                 }
             }
         }
@@ -935,7 +954,7 @@ k_tc_table_batch(const uint8_t* __restrict__ A_hi, const uint8_t* __restrict__ A
         int cnt0 = 0, cnt1 = 0, items = 0;  // tiles issued per stream
         bool ok = true;
         for (int w = blockIdx.x; w < total && ok && !*abort_flag; w += gridDim.x, ++items) {
-            if (!mbar_wait(afull, (uint32_t)items & 1u, global_ns() + TC_TIMEOUT_NS)) {
+            if (!mbar_wait(afull, (uint32_t)items & 1u)) {
                 fail();
                 break;
             }
@@ -948,7 +967,7 @@ k_tc_table_batch(const uint8_t* __restrict__ A_hi, const uint8_t* __restrict__ A
                 const uint32_t idesc = (1u << 4) | (TcFmt<FMT>::atype << 7) | (TcFmt<FMT>::atype << 10) |
                                        ((uint32_t)(Nt >> 3) << 17) | ((uint32_t)(TC_BM >> 4) << 24);
                 const int cs = s ? cnt1 : cnt0;
-                if (cs >= 1 && !mbar_wait(&tempty[s], (uint32_t)(cs - 1) & 1u, global_ns() + TC_TIMEOUT_NS)) {
+                if (cs >= 1 && !mbar_wait(&tempty[s], (uint32_t)(cs - 1) & 1u)) {
                     fail();
                     ok = false;
                     break;
@@ -957,7 +976,7 @@ k_tc_table_batch(const uint8_t* __restrict__ A_hi, const uint8_t* __restrict__ A
                 const uint32_t acc0 = tmem + (uint32_t)s * kAcc;
                 for (int c = 0; c < KC; ++c, ++gb, rs = rs + 1 == stages ? (rp ^= 1u, 0) : rs + 1) {
                     const int st = rs;
-                    if (!mbar_wait(&full[st], rp, global_ns() + TC_TIMEOUT_NS)) {
+                    if (!mbar_wait(&full[st], rp)) {
                         fail();
                         ok = false;
                         break;
@@ -966,11 +985,10 @@ k_tc_table_batch(const uint8_t* __restrict__ A_hi, const uint8_t* __restrict__ A
                     const uint32_t sa = smem_u32(apanel + (size_t)c * kAChunk);
                     const uint32_t sa_lo = sa + kABytes;
                     const uint32_t sb = smem_u32(bring + (size_t)st * kBStage);
-                    const uint32_t sb_lo = sb + kBBytes;
                     // descriptors of the chunk's first K step; a step of 16 elements (256 B) adds 16 to the
                     // address field (addresses stay below 2^18, so no carry leaves the 14-bit field)
                     const uint64_t dA0 = smem_desc(sa, kSbo), dB0 = smem_desc(sb, kSbo);
-                    const uint64_t dAl0 = smem_desc(sa_lo, kSbo), dBl0 = smem_desc(sb_lo, kSbo);
+                    const uint64_t dAl0 = smem_desc(sa_lo, kSbo);
 #pragma unroll
                     for (int ks = 0; ks < (int)TcFmt<FMT>::mmas; ++ks) {
                         if (c == KC - 1 && ks >= klast) break;  // the last chunk's zero K steps
@@ -978,11 +996,7 @@ k_tc_table_batch(const uint8_t* __restrict__ A_hi, const uint8_t* __restrict__ A
                         const uint32_t acc = (c > 0 || ks > 0) ? 1u : 0u;
                         const uint64_t kd = (uint64_t)(ko >> 4);
                         const uint64_t da = dA0 + kd, db = dB0 + kd;
-                        mma_issue<FMT>(acc0, da, db, idesc, acc);
-                        if (SPLIT) {
-                            mma_issue<FMT>(acc0 + 128, da, dBl0 + kd, idesc, acc);
-                            mma_issue<FMT>(acc0 + 128, dAl0 + kd, db, idesc, 1u);
-                        }
+                        mma_step<FMT>(acc0, Nt, da, dAl0 + kd, db, idesc, acc);
                     }
                     mma_commit(&empty[st]);
                 }
@@ -1002,6 +1016,7 @@ k_tc_table_batch(const uint8_t* __restrict__ A_hi, const uint8_t* __restrict__ A
         const int cb0 = half * (TC_BN / 2);
         const int row = qw4 * 32 + lane;
         uint64_t* xb = &xbar[sme * 4 + qw4];
+        constexpr uint32_t kXch = SPLIT ? kAcc - 32 : TC_BN / 2;
         int cnt = 0, nx = 0;
         bool ok = true;
         float z[KT];
@@ -1040,7 +1055,7 @@ k_tc_table_batch(const uint8_t* __restrict__ A_hi, const uint8_t* __restrict__ A
                     cbl[c2] = cok ? -2.f * d.q_scale[col] : 0.f;
                     nbl[c2] = cok ? d.qnorm[col] : 0.f;
                 }
-                if (!mbar_wait(&tfull[sme], (uint32_t)cnt & 1u, global_ns() + TC_TIMEOUT_NS)) {
+                if (!mbar_wait(&tfull[sme], (uint32_t)cnt & 1u)) {
                     fail();
                     ok = false;
                     break;
@@ -1052,7 +1067,7 @@ k_tc_table_batch(const uint8_t* __restrict__ A_hi, const uint8_t* __restrict__ A
                     if (cb0 + cc < Nt) {
                         uint32_t r0[16], r1[16];
                         tmem_ld16(tbase + (uint32_t)(cb0 + cc), r0);
-                        if (SPLIT) tmem_ld16(tbase + 128u + (uint32_t)(cb0 + cc), r1);
+                        if (SPLIT) tmem_ld16(tbase + (uint32_t)Nt + (uint32_t)(cb0 + cc), r1);
                         tmem_wait_ld();
 #pragma unroll
                         for (int e = 0; e < 16; ++e) {
@@ -1071,7 +1086,8 @@ k_tc_table_batch(const uint8_t* __restrict__ A_hi, const uint8_t* __restrict__ A
                 const bool last = n0 + TC_BN >= N;
                 if (last && N > TC_BN / 2) {
                     // the query's last tile: the upper half hands its list to the lower half
-                    // through its own (already drained) TMEM columns cb0 .. cb0 + 31
+                    // through TMEM columns that only it reads (and has drained) or nobody uses: the
+                    // buffer's last 32 (split: the cross terms of columns 96..127, or past 2 Nt)
                     if (half == 1) {
                         uint32_t x[32];
 #pragma unroll
@@ -1079,19 +1095,19 @@ k_tc_table_batch(const uint8_t* __restrict__ A_hi, const uint8_t* __restrict__ A
                             x[l] = __float_as_uint(l < KT ? z[l < KT ? l : 0] : INFINITY);
                             x[16 + l] = (uint32_t)(l < KT ? sj[l < KT ? l : 0] : INT32_MAX);
                         }
-                        tmem_st32(tbase + (uint32_t)cb0, x);
+                        tmem_st32(tbase + kXch, x);
                         tmem_wait_st();
                         tc_fence_before();
                         __syncwarp();
                         if (lane == 0) mbar_arrive(xb);
                     } else {
-                        if (!mbar_wait(xb, (uint32_t)nx & 1u, global_ns() + TC_TIMEOUT_NS)) {
+                        if (!mbar_wait(xb, (uint32_t)nx & 1u)) {
                             fail();
                             ok = false;
                         } else {
                             tc_fence_after();
                             uint32_t x[32];
-                            tmem_ld32(tbase + (uint32_t)(TC_BN / 2), x);
+                            tmem_ld32(tbase + kXch, x);
                             tmem_wait_ld();
 #pragma unroll
                             for (int l = 0; l < KT; ++l)
@@ -1203,6 +1219,11 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity
     while (!mbar_try_wait_cluster(bar, parity))
         if (global_ns() > deadline) return false;
     return true;
+}
+
+__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity)
+{
+    return mbar_try_wait_cluster(bar, parity) || mbar_wait_cluster(bar, parity, global_ns() + TC_TIMEOUT_NS);
 }
 
 __device__ __forceinline__ void tmem_alloc_pair(uint32_t* slot, uint32_t ncols)
@@ -1326,7 +1347,7 @@ k_tc_table_pair(const uint8_t* __restrict__ A_hi, const uint8_t* __restrict__ A_
         bool ok = true;
         for (int w = cid; w < total && ok && !*abort_flag; w += ncl, ++items) {
             const int64_t m0 = (int64_t)(w % pairs) * (2 * TC_BM) + (int64_t)rank * TC_BM;
-            if (items > 0 && !mbar_wait_cluster(afree, (uint32_t)(items - 1) & 1u, global_ns() + TC_TIMEOUT_NS)) {
+            if (items > 0 && !mbar_wait_cluster(afree, (uint32_t)(items - 1) & 1u)) {
                 fail();
                 break;
             }
@@ -1350,8 +1371,7 @@ k_tc_table_pair(const uint8_t* __restrict__ A_hi, const uint8_t* __restrict__ A_
                 const uint8_t* bl = static_cast<const uint8_t*>(d.q_lo);
                 for (int c = 0; c < KC; ++c, ++gb, rs = rs + 1 == stages ? (rp ^= 1u, 0) : rs + 1) {
                     const int st = rs;
-                    if (gb >= stages && !mbar_wait_cluster(&empty[st], rp ^ 1u,
-                                                           global_ns() + TC_TIMEOUT_NS)) {
+                    if (gb >= stages && !mbar_wait_cluster(&empty[st], rp ^ 1u)) {
                         fail();
                         ok = false;
                         break;
@@ -1376,7 +1396,7 @@ k_tc_table_pair(const uint8_t* __restrict__ A_hi, const uint8_t* __restrict__ A_
         int items = 0;
         bool ok = true;
         for (int w = cid; w < total && ok && !*abort_flag; w += ncl, ++items) {
-            if (!mbar_wait(afull, (uint32_t)items & 1u, global_ns() + TC_TIMEOUT_NS)) {
+            if (!mbar_wait(afull, (uint32_t)items & 1u)) {
                 fail();
                 break;
             }
@@ -1388,7 +1408,7 @@ k_tc_table_pair(const uint8_t* __restrict__ A_hi, const uint8_t* __restrict__ A_
             while (ok && ts.next(qd, q, n0, s)) {
                 for (int c = 0; c < KC; ++c, ++gb, rs = rs + 1 == stages ? (rp ^= 1u, 0) : rs + 1) {
                     const int st = rs;
-                    if (!mbar_wait(&full[st], rp, global_ns() + TC_TIMEOUT_NS)) {
+                    if (!mbar_wait(&full[st], rp)) {
                         fail();
                         ok = false;
                         break;
@@ -1404,8 +1424,8 @@ k_tc_table_pair(const uint8_t* __restrict__ A_hi, const uint8_t* __restrict__ A_
         int cnt0 = 0, cnt1 = 0, items = 0;  // tiles issued per stream
         bool ok = true;
         for (int w = cid; w < total && ok && !*abort_flag; w += ncl, ++items) {
-            if (!mbar_wait(afull, (uint32_t)items & 1u, global_ns() + TC_TIMEOUT_NS) ||
-                !mbar_wait_cluster(pafull, (uint32_t)items & 1u, global_ns() + TC_TIMEOUT_NS)) {
+            if (!mbar_wait(afull, (uint32_t)items & 1u) ||
+                !mbar_wait_cluster(pafull, (uint32_t)items & 1u)) {
                 fail();
                 break;
             }
@@ -1418,7 +1438,7 @@ k_tc_table_pair(const uint8_t* __restrict__ A_hi, const uint8_t* __restrict__ A_
                 const uint32_t idesc = (1u << 4) | ((uint32_t)(Nt >> 3) << 17) | ((uint32_t)((2 * TC_BM) >> 4) << 24);
                 const int cs = s ? cnt1 : cnt0;
                 if (cs >= 1 &&
-                    !mbar_wait_cluster(&tempty[s], (uint32_t)(cs - 1) & 1u, global_ns() + TC_TIMEOUT_NS)) {
+                    !mbar_wait_cluster(&tempty[s], (uint32_t)(cs - 1) & 1u)) {
                     fail();
                     ok = false;
                     break;
@@ -1427,8 +1447,8 @@ k_tc_table_pair(const uint8_t* __restrict__ A_hi, const uint8_t* __restrict__ A_
                 const uint32_t acc0 = tmem + (uint32_t)s * kAcc;
                 for (int c = 0; c < KC; ++c, ++gb, rs = rs + 1 == stages ? (rp ^= 1u, 0) : rs + 1) {
                     const int st = rs;
-                    if (!mbar_wait(&full[st], rp, global_ns() + TC_TIMEOUT_NS) ||
-                        !mbar_wait_cluster(&pfull[st], rp, global_ns() + TC_TIMEOUT_NS)) {
+                    if (!mbar_wait(&full[st], rp) ||
+                        !mbar_wait_cluster(&pfull[st], rp)) {
                         fail();
                         ok = false;
                         break;
@@ -1505,7 +1525,7 @@ k_tc_table_pair(const uint8_t* __restrict__ A_hi, const uint8_t* __restrict__ A_
                     cbl[c4] = cok ? -2.f * d.q_scale[col] : 0.f;
                     nbl[c4] = cok ? d.qnorm[col] : 0.f;
                 }
-                if (!mbar_wait_cluster(&tfull[sme], (uint32_t)cnt & 1u, global_ns() + TC_TIMEOUT_NS)) {
+                if (!mbar_wait_cluster(&tfull[sme], (uint32_t)cnt & 1u)) {
                     fail();
                     ok = false;
                     break;
@@ -1643,7 +1663,7 @@ k_tc_cand_batch(const QDesc* __restrict__ qd, const int* __restrict__ nq_dev, in
             if (item_rows(w) == 0) continue;
             const QDesc& d = qd[w / kRT];
             const int64_t m0 = (int64_t)(w % kRT) * TC_BM;
-            if (items > 0 && !mbar_wait(afree, (uint32_t)(items - 1) & 1u, global_ns() + TC_TIMEOUT_NS)) {
+            if (items > 0 && !mbar_wait(afree, (uint32_t)(items - 1) & 1u)) {
                 fail();
                 break;
             }
@@ -1664,7 +1684,7 @@ k_tc_cand_batch(const QDesc* __restrict__ qd, const int* __restrict__ nq_dev, in
                 for (int c = 0; c < KC; ++c, ++gb, rs = rs + 1 == stages ? (rp ^= 1u, 0) : rs + 1) {
                     const int s = rs;
                     if (gb >= stages &&
-                        !mbar_wait(&empty[s], rp ^ 1u, global_ns() + TC_TIMEOUT_NS)) {
+                        !mbar_wait(&empty[s], rp ^ 1u)) {
                         fail();
                         ok = false;
                         break;
@@ -1672,7 +1692,7 @@ k_tc_cand_batch(const QDesc* __restrict__ qd, const int* __restrict__ nq_dev, in
                     uint8_t* bst = bring + (size_t)s * kBStage;
                     mbar_expect_tx(&full[s], (uint32_t)kParts * b_bytes);
                     bulk_g2s(bst, bh + ((int64_t)c * d.npad + n0) * EB, b_bytes, &full[s]);
-                    if (SPLIT) bulk_g2s(bst + kBBytes, bl + ((int64_t)c * d.npad + n0) * EB, b_bytes, &full[s]);
+                    if (SPLIT) bulk_g2s(bst + b_bytes, bl + ((int64_t)c * d.npad + n0) * EB, b_bytes, &full[s]);
                 }
             }
         }
@@ -1689,7 +1709,7 @@ k_tc_cand_batch(const QDesc* __restrict__ qd, const int* __restrict__ nq_dev, in
         for (int w = blockIdx.x; w < total && ok && !*abort_flag; w += gridDim.x) {
             if (item_rows(w) == 0) continue;
             const int h = qd[w / kRT].h;
-            if (!mbar_wait(afull, (uint32_t)items & 1u, global_ns() + TC_TIMEOUT_NS)) {
+            if (!mbar_wait(afull, (uint32_t)items & 1u)) {
                 fail();
                 break;
             }
@@ -1699,7 +1719,7 @@ k_tc_cand_batch(const QDesc* __restrict__ qd, const int* __restrict__ nq_dev, in
                 const uint32_t idesc = (1u << 4) | (TcFmt<FMT>::atype << 7) | (TcFmt<FMT>::atype << 10) |
                                        ((uint32_t)(Nt >> 3) << 17) | ((uint32_t)(TC_BM >> 4) << 24);
                 const int buf = it & 1;
-                if (it >= 2 && !mbar_wait(&tempty[buf], (uint32_t)((it >> 1) - 1) & 1u, global_ns() + TC_TIMEOUT_NS)) {
+                if (it >= 2 && !mbar_wait(&tempty[buf], (uint32_t)((it >> 1) - 1) & 1u)) {
                     fail();
                     ok = false;
                     break;
@@ -1708,7 +1728,7 @@ k_tc_cand_batch(const QDesc* __restrict__ qd, const int* __restrict__ nq_dev, in
                 const uint32_t acc0 = tmem + (uint32_t)buf * kAcc;
                 for (int c = 0; c < KC; ++c, ++gb, rs = rs + 1 == stages ? (rp ^= 1u, 0) : rs + 1) {
                     const int s = rs;
-                    if (!mbar_wait(&full[s], rp, global_ns() + TC_TIMEOUT_NS)) {
+                    if (!mbar_wait(&full[s], rp)) {
                         fail();
                         ok = false;
                         break;
@@ -1717,22 +1737,17 @@ k_tc_cand_batch(const QDesc* __restrict__ qd, const int* __restrict__ nq_dev, in
                     const uint32_t sa = smem_u32(apanel + (size_t)c * kAChunk);
                     const uint32_t sa_lo = sa + kABytes;
                     const uint32_t sb = smem_u32(bring + (size_t)s * kBStage);
-                    const uint32_t sb_lo = sb + kBBytes;
                     // descriptors of the chunk's first K step; a step of 16 elements (256 B) adds 16 to the
                     // address field (addresses stay below 2^18, so no carry leaves the 14-bit field)
                     const uint64_t dA0 = smem_desc(sa, kSbo), dB0 = smem_desc(sb, kSbo);
-                    const uint64_t dAl0 = smem_desc(sa_lo, kSbo), dBl0 = smem_desc(sb_lo, kSbo);
+                    const uint64_t dAl0 = smem_desc(sa_lo, kSbo);
 #pragma unroll
                     for (int ks = 0; ks < (int)TcFmt<FMT>::mmas; ++ks) {
                         const uint32_t ko = (uint32_t)ks * 256u;
                         const uint32_t acc = (c > 0 || ks > 0) ? 1u : 0u;
                         const uint64_t kd = (uint64_t)(ko >> 4);
                         const uint64_t da = dA0 + kd, db = dB0 + kd;
-                        mma_issue<FMT>(acc0, da, db, idesc, acc);
-                        if (SPLIT) {
-                            mma_issue<FMT>(acc0 + 128, da, dBl0 + kd, idesc, acc);
-                            mma_issue<FMT>(acc0 + 128, dAl0 + kd, db, idesc, 1u);
-                        }
+                        mma_step<FMT>(acc0, Nt, da, dAl0 + kd, db, idesc, acc);
                     }
                     mma_commit(&empty[s]);
                 }
@@ -1763,7 +1778,7 @@ k_tc_cand_batch(const QDesc* __restrict__ qd, const int* __restrict__ nq_dev, in
                 const bool lok = lcol < N;
                 const float cb_l = lok ? -2.f * d.qs_scale[lcol] : 0.f;
                 const float nb_l = lok ? d.qnorm[lcol] : 0.f;
-                if (!mbar_wait(&tfull[buf], (uint32_t)(it >> 1) & 1u, global_ns() + TC_TIMEOUT_NS)) {
+                if (!mbar_wait(&tfull[buf], (uint32_t)(it >> 1) & 1u)) {
                     fail();
                     ok = false;
                     break;
@@ -1776,7 +1791,7 @@ k_tc_cand_batch(const QDesc* __restrict__ qd, const int* __restrict__ nq_dev, in
                     for (int hh = 0; hh < 2; ++hh) {
                         uint32_t r0[16], r1[16];
                         tmem_ld16(tbase + (uint32_t)(cc + 16 * hh), r0);
-                        if (SPLIT) tmem_ld16(tbase + 128u + (uint32_t)(cc + 16 * hh), r1);
+                        if (SPLIT) tmem_ld16(tbase + (uint32_t)Nt + (uint32_t)(cc + 16 * hh), r1);
                         tmem_wait_ld();
 #pragma unroll
                         for (int e4 = 4 * hh; e4 < 4 * hh + 4; ++e4) {
