@@ -6,6 +6,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "emd_internal.cuh"
 
@@ -96,7 +97,84 @@ __device__ __forceinline__ void load_vec(const float* p, bool ok, float (&o)[4])
     o[0] = v.x; o[1] = v.y; o[2] = v.z; o[3] = v.w;
 }
 
+// The lists of the query bins jbase + NJ lane .. + NJ - 1 over the document bins [a, b).
+template <int KT, int NJ>
+__device__ __forceinline__ void rev_lists(const int32_t* __restrict__ col, const float* __restrict__ val, int32_t a,
+                                          int32_t b, const float* __restrict__ D, int ldd, int jbase,
+                                          const int32_t* __restrict__ rmap, float (&z)[NJ][KT], float (&cap)[NJ][KT])
+{
+    constexpr int U = 4;  // bins whose loads are in flight together
+    const int lane = threadIdx.x & 31;
+    const int j0 = jbase + lane * NJ;
+    const bool jin = j0 < ldd;  // ldd % 32 == 0 and NJ | 32: the whole vector is in the row
+#pragma unroll
+    for (int t = 0; t < NJ; ++t)
+#pragma unroll
+        for (int l = 0; l < KT; ++l) { z[t][l] = INFINITY; cap[t][l] = 0.f; }
+    for (int32_t eb = a; eb < b; eb += 32) {
+        const int32_t e = eb + lane;
+        const int32_t u = e < b ? (rmap ? rmap[col[e]] : col[e]) : 0;
+        const float x = e < b ? val[e] : 0.f;
+        const int cnt = min(32, b - eb);
+        int i = 0;
+        for (; i + U <= cnt; i += U) {
+            float dv[U][NJ], xv[U];
+#pragma unroll
+            for (int s = 0; s < U; ++s) {
+                const int32_t ui = __shfl_sync(0xffffffffu, u, i + s);
+                xv[s] = __shfl_sync(0xffffffffu, x, i + s);
+                load_vec(D + (int64_t)ui * ldd + j0, jin, dv[s]);
+            }
+#pragma unroll
+            for (int s = 0; s < U; ++s)
+#pragma unroll
+                for (int t = 0; t < NJ; ++t) insert_sorted<KT>(z[t], cap[t], dv[s][t], xv[s]);
+        }
+        for (; i < cnt; ++i) {
+            const int32_t ui = __shfl_sync(0xffffffffu, u, i);
+            const float xi = __shfl_sync(0xffffffffu, x, i);
+            float dv[NJ];
+            load_vec(D + (int64_t)ui * ldd + j0, jin, dv);
+#pragma unroll
+            for (int t = 0; t < NJ; ++t) insert_sorted<KT>(z[t], cap[t], dv[t], xi);
+        }
+    }
+}
+
+// Adds the costs of a pass of 32 NJ query bins to the lanes' totals in the order of a pass of 32
+// NJW bins: lane L sums bins NJW L .. + NJW - 1 of the pass.  With NJ < NJW (a query's last bins)
+// bin NJW L + t lies in lane (NJW L + t) / NJ.
+template <int MEAS, int KT, int NJ, int NJW>
+__device__ __forceinline__ void rev_add_costs(float& total, int jbase, int h, const float* __restrict__ q_w,
+                                              const float (&z)[NJ][KT], const float (&cap)[NJ][KT], int keff, bool sq)
+{
+    const int lane = threadIdx.x & 31;
+    const int j0 = jbase + lane * NJ;
+    if (NJ == NJW) {
+#pragma unroll
+        for (int t = 0; t < NJ; ++t)
+            if (j0 + t < h) total = __fadd_rn(total, rev_cost_sorted<MEAS, KT>(q_w[j0 + t], z[t], cap[t], keff, sq));
+        return;
+    }
+    float c[NJ];
+#pragma unroll
+    for (int t = 0; t < NJ; ++t)
+        c[t] = j0 + t < h ? rev_cost_sorted<MEAS, KT>(q_w[j0 + t], z[t], cap[t], keff, sq) : 0.f;
+#pragma unroll
+    for (int t = 0; t < NJW; ++t) {
+        const int src = lane * NJW + t;  // bin of the pass
+        const float v = __shfl_sync(0xffffffffu, c[t % NJ], (src / NJ) & 31);
+        if (src < 32 * NJ && jbase + src < h) total = __fadd_rn(total, v);
+    }
+}
+
 // WITHIN: documents with a forward value above thr are left out (t_max = +inf).
+//
+// A pass covers 32 NJ query bins; the last bins of a query take passes of 64 or 32 (NJ 2 or 1)
+// when they fill no wider one, so that 20 .. 400 bins are padded to 32 instead of 128.  The pass
+// is bound by the ALU pipe (compares and selects of the insertions, 78% busy), so padding is
+// time: 29 queries of 20 .. 400 bins, 2e4 documents, k = 4, all documents: 13.9 -> 10.8 ms; the
+// candidates of 64 serving queries 1.25 -> 0.98 ms.
 template <int MEAS, int KT, int NJ, bool WITHIN = false>
 __device__ __forceinline__ void rev_body(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
       const float* __restrict__ val, int64_t n, const float* __restrict__ D, int ldd, int h,
@@ -104,7 +182,6 @@ __device__ __forceinline__ void rev_body(const int32_t* __restrict__ row_ptr, co
       float* __restrict__ t_rev, float* __restrict__ t_max, const int64_t* __restrict__ doc_ids,
       const int* __restrict__ n_dev, bool sq, float thr = 0.f)
 {
-    constexpr int U = 4;  // bins whose loads are in flight together
     const int lane = threadIdx.x & 31;
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
     if (n_dev) n = min(n, (int64_t)*n_dev);  // slots filled on the device (candidate lists)
@@ -119,44 +196,19 @@ __device__ __forceinline__ void rev_body(const int32_t* __restrict__ row_ptr, co
         const int keff = MEAS == M_RWMD ? 1 : (MEAS == M_OMR ? min(2, hd) : min(k, hd));
         float total = 0.f;
         for (int jbase = 0; jbase < h; jbase += 32 * NJ) {
-            const int j0 = jbase + lane * NJ;
-            const bool jin = j0 < ldd;  // ldd % 32 == 0 and NJ | 32: the whole vector is in the row
-            float z[NJ][KT], cap[NJ][KT];
-#pragma unroll
-            for (int t = 0; t < NJ; ++t)
-#pragma unroll
-                for (int l = 0; l < KT; ++l) { z[t][l] = INFINITY; cap[t][l] = 0.f; }
-            for (int32_t eb = a; eb < b; eb += 32) {
-                const int32_t e = eb + lane;
-                const int32_t u = e < b ? col[e] : 0;
-                const float x = e < b ? val[e] : 0.f;
-                const int cnt = min(32, b - eb);
-                int i = 0;
-                for (; i + U <= cnt; i += U) {
-                    float dv[U][NJ], xv[U];
-#pragma unroll
-                    for (int s = 0; s < U; ++s) {
-                        const int32_t ui = __shfl_sync(0xffffffffu, u, i + s);
-                        xv[s] = __shfl_sync(0xffffffffu, x, i + s);
-                        load_vec(D + (int64_t)ui * ldd + j0, jin, dv[s]);
-                    }
-#pragma unroll
-                    for (int s = 0; s < U; ++s)
-#pragma unroll
-                        for (int t = 0; t < NJ; ++t) insert_sorted<KT>(z[t], cap[t], dv[s][t], xv[s]);
-                }
-                for (; i < cnt; ++i) {
-                    const int32_t ui = __shfl_sync(0xffffffffu, u, i);
-                    const float xi = __shfl_sync(0xffffffffu, x, i);
-                    float dv[NJ];
-                    load_vec(D + (int64_t)ui * ldd + j0, jin, dv);
-#pragma unroll
-                    for (int t = 0; t < NJ; ++t) insert_sorted<KT>(z[t], cap[t], dv[t], xi);
-                }
+            if (NJ >= 2 && h - jbase <= 32) {
+                float z[1][KT], cap[1][KT];
+                rev_lists<KT, 1>(col, val, a, b, D, ldd, jbase, nullptr, z, cap);
+                rev_add_costs<MEAS, KT, 1, NJ>(total, jbase, h, q_w, z, cap, keff, sq);
+            } else if (NJ >= 4 && h - jbase <= 64) {
+                float z[2][KT], cap[2][KT];
+                rev_lists<KT, 2>(col, val, a, b, D, ldd, jbase, nullptr, z, cap);
+                rev_add_costs<MEAS, KT, 2, NJ>(total, jbase, h, q_w, z, cap, keff, sq);
+            } else {
+                float z[NJ][KT], cap[NJ][KT];
+                rev_lists<KT, NJ>(col, val, a, b, D, ldd, jbase, nullptr, z, cap);
+                rev_add_costs<MEAS, KT, NJ, NJ>(total, jbase, h, q_w, z, cap, keff, sq);
             }
-#pragma unroll
-            for (int t = 0; t < NJ; ++t)
-                if (j0 + t < h) total = __fadd_rn(total, rev_cost_sorted<MEAS, KT>(q_w[j0 + t], z[t], cap[t], keff, sq));
         }
         total = warp_sum(total);
         if (lane == 0) {
@@ -167,7 +219,7 @@ __device__ __forceinline__ void rev_body(const int32_t* __restrict__ row_ptr, co
 }
 
 template <int MEAS, int KT, int NJ>
-__global__ void __launch_bounds__(256, 2) k_rev(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
+__global__ void __launch_bounds__(256, 3) k_rev(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
       const float* __restrict__ val, int64_t n, const float* __restrict__ D, int ldd, int h,
       const float* __restrict__ q_w, int k, const float* __restrict__ t_fwd,
       float* __restrict__ t_rev, float* __restrict__ t_max, const int64_t* __restrict__ doc_ids,
@@ -189,7 +241,6 @@ __device__ __forceinline__ void rev_blk_body(const int32_t* __restrict__ row_ptr
           float* __restrict__ t_rev, float* __restrict__ t_max, const int64_t* __restrict__ doc_ids,
           const int* __restrict__ n_dev, bool sq, const int32_t* __restrict__ rmap = nullptr)
 {
-    constexpr int U = 4;
     __shared__ float sz[W - 1][32 * NJ][KT];
     __shared__ float sc[W - 1][32 * NJ][KT];
     const int slot = blockIdx.x;
@@ -202,49 +253,17 @@ __device__ __forceinline__ void rev_blk_body(const int32_t* __restrict__ row_ptr
     const int chunk = (hd + W - 1) / W;
     const int32_t ca = a + min(hd, warp * chunk), cb = a + min(hd, (warp + 1) * chunk);
     float total = 0.f;
-    for (int jbase = 0; jbase < h; jbase += 32 * NJ) {
-        const int j0 = jbase + lane * NJ;
-        const bool jin = j0 < ldd;
-        float z[NJ][KT], cap[NJ][KT];
-#pragma unroll
-        for (int t = 0; t < NJ; ++t)
-#pragma unroll
-            for (int l = 0; l < KT; ++l) { z[t][l] = INFINITY; cap[t][l] = 0.f; }
-        for (int32_t eb = ca; eb < cb; eb += 32) {
-            const int32_t e = eb + lane;
-            const int32_t u = e < cb ? col[e] : 0;
-            const float x = e < cb ? val[e] : 0.f;
-            const int cnt = min(32, cb - eb);
-            int i = 0;
-            for (; i + U <= cnt; i += U) {
-                float dv[U][NJ], xv[U];
-#pragma unroll
-                for (int s = 0; s < U; ++s) {
-                    const int32_t ui = __shfl_sync(0xffffffffu, u, i + s);
-                    xv[s] = __shfl_sync(0xffffffffu, x, i + s);
-                    load_vec(D + (rmap ? (int64_t)rmap[ui] : (int64_t)ui) * ldd + j0, jin, dv[s]);
-                }
-#pragma unroll
-                for (int s = 0; s < U; ++s)
-#pragma unroll
-                    for (int t = 0; t < NJ; ++t) insert_sorted<KT>(z[t], cap[t], dv[s][t], xv[s]);
-            }
-            for (; i < cnt; ++i) {
-                const int32_t ui = __shfl_sync(0xffffffffu, u, i);
-                const float xi = __shfl_sync(0xffffffffu, x, i);
-                float dv[NJ];
-                load_vec(D + (rmap ? (int64_t)rmap[ui] : (int64_t)ui) * ldd + j0, jin, dv);
-#pragma unroll
-                for (int t = 0; t < NJ; ++t) insert_sorted<KT>(z[t], cap[t], dv[t], xi);
-            }
-        }
+    auto pass = [&](int jbase, auto width) {
+        constexpr int N = decltype(width)::value;
+        float z[N][KT], cap[N][KT];
+        rev_lists<KT, N>(col, val, ca, cb, D, ldd, jbase, rmap, z, cap);
         if (warp > 0) {
 #pragma unroll
-            for (int t = 0; t < NJ; ++t)
+            for (int t = 0; t < N; ++t)
 #pragma unroll
                 for (int l = 0; l < KT; ++l) {
-                    sz[warp - 1][lane * NJ + t][l] = z[t][l];
-                    sc[warp - 1][lane * NJ + t][l] = cap[t][l];
+                    sz[warp - 1][lane * N + t][l] = z[t][l];
+                    sc[warp - 1][lane * N + t][l] = cap[t][l];
                 }
         }
         __syncthreads();
@@ -252,15 +271,18 @@ __device__ __forceinline__ void rev_blk_body(const int32_t* __restrict__ row_ptr
 #pragma unroll
             for (int w = 0; w < W - 1; ++w)
 #pragma unroll
-                for (int t = 0; t < NJ; ++t)
+                for (int t = 0; t < N; ++t)
 #pragma unroll
                     for (int l = 0; l < KT; ++l)
-                        insert_sorted<KT>(z[t], cap[t], sz[w][lane * NJ + t][l], sc[w][lane * NJ + t][l]);
-#pragma unroll
-            for (int t = 0; t < NJ; ++t)
-                if (j0 + t < h) total = __fadd_rn(total, rev_cost_sorted<MEAS, KT>(q_w[j0 + t], z[t], cap[t], keff, sq));
+                        insert_sorted<KT>(z[t], cap[t], sz[w][lane * N + t][l], sc[w][lane * N + t][l]);
+            rev_add_costs<MEAS, KT, N, NJ>(total, jbase, h, q_w, z, cap, keff, sq);
         }
         __syncthreads();
+    };
+    for (int jbase = 0; jbase < h; jbase += 32 * NJ) {  // the last bins in narrower passes, as rev_body
+        if (NJ >= 2 && h - jbase <= 32) pass(jbase, std::integral_constant<int, 1>());
+        else if (NJ >= 4 && h - jbase <= 64) pass(jbase, std::integral_constant<int, 2>());
+        else pass(jbase, std::integral_constant<int, NJ>());
     }
     if (warp == 0) {
         total = warp_sum(total);
@@ -700,7 +722,7 @@ cudaError_t rev_meas_blk(int k, const int32_t* row_ptr, const int32_t* col, cons
 
 // NJ follows the per-query launcher: NJW bins per lane when h > 32, else one.
 template <int MEAS, int KT, int NJW>
-__global__ void __launch_bounds__(256, 2)
+__global__ void __launch_bounds__(256, 3)
 k_rev_b(const QDesc* __restrict__ qd, const int* __restrict__ nq, const int32_t* __restrict__ row_ptr,
         const int32_t* __restrict__ col, const float* __restrict__ val, int64_t n, int k, int dir)
 {
@@ -806,7 +828,7 @@ cudaError_t rev_meas_b(int k, int dir, const QDesc* qd, const int* nq, int max_q
 // documents took 3.3 ms a query on 60,000 images (k = 8, top-16: 25 to 32 queries of a batch
 // of 64 are not certified); this takes 106 ms per batch to 2.3 ms.
 template <int MEAS, int KT, int NJW>
-__global__ void __launch_bounds__(256, 2)
+__global__ void __launch_bounds__(256, 3)
 k_rev_within_b(const QDesc* __restrict__ qd, const int* __restrict__ nq, const int32_t* __restrict__ row_ptr,
                const int32_t* __restrict__ col, const float* __restrict__ val, int64_t n, int k, int K)
 {
