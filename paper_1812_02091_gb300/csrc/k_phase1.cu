@@ -57,35 +57,42 @@ __global__ void k_gather_rows(const float* __restrict__ src, int64_t v, int ld, 
 
 // ------------------------------------------------------------------ FP32 distance tile
 //
-// Block tile 128 (vocabulary rows) x 64 (query columns), K step 16, 128 threads, each
+// Block tile 128 (vocabulary rows) x 64 or 32 (query columns), K step 16, 128 threads, each
 // thread an 8 x 8 register tile (rows tr*4+{0..3} and 64+tr*4+{0..3}, columns tc*4+{0..3}
 // and 32+tc*4+{0..3}).  Both operands are staged k-major in shared memory (double
 // buffered, one barrier per K step) so that the inner loop is 4 LDS.128 + 64 FFMA.
 // Operand rows are zero-padded to a multiple of 4 floats, so the K tail reads zeros.
 
+// BN = 64, or 32 for a query's last columns when at most 32 remain (then 8 x 4 per thread).  The
+// products of two columns share one instruction (f32x2), each rounded as fmaf: FFMA issue
+// slots are halved, which leaves room for the operand reads.  64 text queries (93,255 rows, m =
+// 300): 11.9 -> 10.3 ms, 38 TFLOP/s of the product alone; what bounds it then is the shared-memory
+// data path (90% busy: 16 wavefronts of operand reads to 32 two-column products).
+template <int BN>
 __device__ __forceinline__ void dist_fp32_body(const float* __restrict__ A, int64_t M, int lda, const float* __restrict__ anorm,
             const int32_t* __restrict__ a_ids, const float* __restrict__ B, int N, int ldb,
             const float* __restrict__ bnorm, const int32_t* __restrict__ b_ids, int K,
-            float* __restrict__ D, int ldd)
+            float* __restrict__ D, int ldd, float (*__restrict__ As)[kDistBK][kDistBM],
+            float (*__restrict__ Bs)[kDistBK][kDistBN])
 {
-    constexpr int BM = kDistBM, BN = kDistBN, BK = kDistBK;
-    __shared__ __align__(16) float As[2][BK][BM];
-    __shared__ __align__(16) float Bs[2][BK][BN];
+    constexpr int BM = kDistBM, BK = kDistBK;
+    constexpr int JH = BN / 32;  // column groups of 4 per thread
 
     const int tid = threadIdx.x;
     const int64_t m0 = (int64_t)blockIdx.x * BM;
-    const int n0 = blockIdx.y * BN;
+    const int n0 = blockIdx.y * kDistBN;
     const int tr = tid >> 3, tc = tid & 7;
 
-    // loader mapping: A row tid (16 floats); B row tid>>1, half (tid&1)
+    // loader mapping: A row tid (16 floats); B row tid / (128 / BN), 16 BN / 128 floats of it
+    constexpr int TB = 128 / BN, QB = 4 / TB;
     const int64_t arow = m0 + tid;
     const bool a_ok = arow < M;
     const float* Ap = A + (a_ok ? arow : 0) * lda;
-    const int brow = n0 + (tid >> 1);
-    const int bk = (tid & 1) * 8;
+    const int brow = n0 + tid / TB;
+    const int bk = tid % TB * (QB * 4);
     const float* Bp = B + (int64_t)brow * ldb;
 
-    float4 ra[4], rb[2];
+    float4 ra[4], rb[QB];
     auto load = [&](int k0) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -94,7 +101,7 @@ __device__ __forceinline__ void dist_fp32_body(const float* __restrict__ A, int6
                                        : make_float4(0.f, 0.f, 0.f, 0.f);
         }
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
+        for (int q = 0; q < QB; ++q) {
             int kk = k0 + bk + q * 4;
             rb[q] = (kk < ldb) ? *reinterpret_cast<const float4*>(Bp + kk)
                                : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -109,19 +116,19 @@ __device__ __forceinline__ void dist_fp32_body(const float* __restrict__ A, int6
             As[buf][q * 4 + 3][tid] = ra[q].w;
         }
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            Bs[buf][bk + q * 4 + 0][tid >> 1] = rb[q].x;
-            Bs[buf][bk + q * 4 + 1][tid >> 1] = rb[q].y;
-            Bs[buf][bk + q * 4 + 2][tid >> 1] = rb[q].z;
-            Bs[buf][bk + q * 4 + 3][tid >> 1] = rb[q].w;
+        for (int q = 0; q < QB; ++q) {
+            Bs[buf][bk + q * 4 + 0][tid / TB] = rb[q].x;
+            Bs[buf][bk + q * 4 + 1][tid / TB] = rb[q].y;
+            Bs[buf][bk + q * 4 + 2][tid / TB] = rb[q].z;
+            Bs[buf][bk + q * 4 + 3][tid / TB] = rb[q].w;
         }
     };
 
-    float acc[8][8];
+    float2 acc[8][2 * JH];
 #pragma unroll
     for (int i = 0; i < 8; ++i)
 #pragma unroll
-        for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
+        for (int j = 0; j < 2 * JH; ++j) acc[i][j] = make_float2(0.f, 0.f);
 
     const int Kpad = (int)round_up(K, BK);
     load(0);
@@ -133,16 +140,20 @@ __device__ __forceinline__ void dist_fp32_body(const float* __restrict__ A, int6
         if (more) load(k0 + BK);
 #pragma unroll
         for (int k = 0; k < BK; ++k) {
-            float4 a0 = *reinterpret_cast<const float4*>(&As[buf][k][tr * 4]);
-            float4 a1 = *reinterpret_cast<const float4*>(&As[buf][k][64 + tr * 4]);
-            float4 b0 = *reinterpret_cast<const float4*>(&Bs[buf][k][tc * 4]);
-            float4 b1 = *reinterpret_cast<const float4*>(&Bs[buf][k][32 + tc * 4]);
-            float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-            float b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+            const float4 a0 = *reinterpret_cast<const float4*>(&As[buf][k][tr * 4]);
+            const float4 a1 = *reinterpret_cast<const float4*>(&As[buf][k][64 + tr * 4]);
+            float2 b[2 * JH];
+#pragma unroll
+            for (int j = 0; j < JH; ++j) {
+                const float4 v = *reinterpret_cast<const float4*>(&Bs[buf][k][j * 32 + tc * 4]);
+                b[2 * j] = make_float2(v.x, v.y);
+                b[2 * j + 1] = make_float2(v.z, v.w);
+            }
+            const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
 #pragma unroll
             for (int i = 0; i < 8; ++i)
 #pragma unroll
-                for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+                for (int j = 0; j < 2 * JH; ++j) acc[i][j] = fma2(make_float2(a[i], a[i]), b[j], acc[i][j]);
         }
         if (more) store(buf ^ 1);
         __syncthreads();
@@ -156,16 +167,17 @@ __device__ __forceinline__ void dist_fp32_body(const float* __restrict__ A, int6
         const float an = anorm[row];
         const int32_t aid = a_ids[row];
 #pragma unroll
-        for (int jh = 0; jh < 2; ++jh) {
+        for (int jh = 0; jh < JH; ++jh) {
             const int col0 = n0 + jh * 32 + tc * 4;
             if (col0 >= ldd) continue;
+            const float av[4] = {acc[i][2 * jh].x, acc[i][2 * jh].y, acc[i][2 * jh + 1].x, acc[i][2 * jh + 1].y};
             float o[4];
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 const int col = col0 + e;
                 float d = INFINITY;
                 if (col < N) {
-                    const float d2 = fmaf(-2.f, acc[i][jh * 4 + e], an + bnorm[col]);
+                    const float d2 = fmaf(-2.f, av[e], an + bnorm[col]);
                     d = (aid == b_ids[col]) ? 0.f : d2;
                 }
                 o[e] = d;
@@ -175,12 +187,26 @@ __device__ __forceinline__ void dist_fp32_body(const float* __restrict__ A, int6
     }
 }
 
-__global__ void __launch_bounds__(128) k_dist_fp32(const float* __restrict__ A, int64_t M, int lda, const float* __restrict__ anorm,
+// The column tile at n0: 64 wide, 32 when no more are left.
+__device__ __forceinline__ void dist_fp32_tile(const float* __restrict__ A, int64_t M, int lda, const float* __restrict__ anorm,
             const int32_t* __restrict__ a_ids, const float* __restrict__ B, int N, int ldb,
             const float* __restrict__ bnorm, const int32_t* __restrict__ b_ids, int K,
             float* __restrict__ D, int ldd)
 {
-    dist_fp32_body(A, M, lda, anorm, a_ids, B, N, ldb, bnorm, b_ids, K, D, ldd);
+    __shared__ __align__(16) float As[2][kDistBK][kDistBM];
+    __shared__ __align__(16) float Bs[2][kDistBK][kDistBN];
+    if (ldd - (int)blockIdx.y * kDistBN > 32)
+        dist_fp32_body<64>(A, M, lda, anorm, a_ids, B, N, ldb, bnorm, b_ids, K, D, ldd, As, Bs);
+    else
+        dist_fp32_body<32>(A, M, lda, anorm, a_ids, B, N, ldb, bnorm, b_ids, K, D, ldd, As, Bs);
+}
+
+__global__ void __launch_bounds__(128, 4) k_dist_fp32(const float* __restrict__ A, int64_t M, int lda, const float* __restrict__ anorm,
+            const int32_t* __restrict__ a_ids, const float* __restrict__ B, int N, int ldb,
+            const float* __restrict__ bnorm, const int32_t* __restrict__ b_ids, int K,
+            float* __restrict__ D, int ldd)
+{
+    dist_fp32_tile(A, M, lda, anorm, a_ids, B, N, ldb, bnorm, b_ids, K, D, ldd);
 }
 
 // ------------------------------------------------------------------ cost-matrix gather
@@ -580,14 +606,14 @@ __global__ void k_gather_rows_b(const QDesc* __restrict__ qd, const int* __restr
     gather_rows_body(src, v, ld, m, d.qidx, d.h, d.qrows, d.Q, d.qnorm, err);
 }
 
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(128, 4)
 k_dist_fp32_b(const QDesc* __restrict__ qd, const int* __restrict__ nq, const float* __restrict__ A, int64_t M,
               int lda, const float* __restrict__ anorm, const int32_t* __restrict__ a_ids, int K)
 {
     if ((int)blockIdx.z >= *nq) return;
     const QDesc& d = qd[blockIdx.z];
     if ((int)blockIdx.y * kDistBN >= d.ldd) return;
-    dist_fp32_body(A, M, lda, anorm, a_ids, d.Q, d.h, lda, d.qnorm, d.qidx, K, d.D, d.ldd);
+    dist_fp32_tile(A, M, lda, anorm, a_ids, d.Q, d.h, lda, d.qnorm, d.qidx, K, d.D, d.ldd);
 }
 
 __global__ void k_dist_gather_b(const QDesc* __restrict__ qd, const int* __restrict__ nq, const float* __restrict__ cost,
