@@ -350,13 +350,17 @@ emd_status run_lanes(emd_db* db, const int64_t* rp, const int32_t* qidx, const f
                      int64_t i1, int meas, int k, int dir, int K, bool pruned, float* out_t, int64_t* out_idx,
                      float* out_dist, cudaStream_t st);
 
-// Whether a sub-batch runs in the fused form (the Phase-1 table from the product's epilogue,
-// reverse distances on the candidate documents' rows only).
+// Whether a sub-batch runs in the fused form: the Phase-1 table from the product's epilogue and no
+// full distance matrix.  Pruned top-K (reverse distances on the candidate documents' rows only),
+// and with FP32_TC the forward direction alone, whose tables are all it needs (the
+// approximate formats' fused tables are certified, their full-matrix ones are not, so they keep
+// the latter).
 bool fused_form(const BatchWS& ws, const emd_db* db, int meas, int k, int dir, bool pruned, bool allow_fused)
 {
-    if (!pruned || !allow_fused || !ws.fused || meas == M_ICT) return false;
+    if (!allow_fused || !ws.fused || meas == M_ICT) return false;
+    if (!pruned && (dir != EMD_DIR_FWD || db->approx)) return false;
     const int H = db->opt.max_query_h;
-    const int tk_b = dir != EMD_DIR_REV ? table_width(db, meas, k, H) : 0;
+    const int tk_b = table_width(db, meas, k, H);
     return tk_b <= 16 && (!db->approx || std::min(rerank_width(db, tk_b, H), kRerankMax) <= kCandPerRow);
 }
 
@@ -377,8 +381,8 @@ emd_status launch_sequence(BatchWS& ws, emd_db* db, int slot, int meas, int k, i
     const int kc_b = db->approx ? std::min(rerank_width(db, tk_b, H), kRerankMax) : tk_b;
     if (!hd && fused_form(ws, db, meas, k, dir, pruned, allow_fused)) {
         // fused form: the table from the product's epilogue (approximate formats: candidates
-        // re-ranked exactly); the reverse direction's distances on the candidate documents' rows
-        // only, exact in the FP16 split
+        // re-ranked exactly); for the pruned top-K the reverse direction's distances on the
+        // candidate documents' rows only, exact in the FP16 split
         {
             Phase p(db, 0, db->approx ? 3 : 2, st);
             const int prow = (int)round_up(H, 128);
@@ -421,9 +425,20 @@ emd_status launch_sequence(BatchWS& ws, emd_db* db, int slot, int meas, int k, i
         }
         {
             Phase p(db, 3, 1, st);
-            EMD_CUDA(launch_fwd_b(meas, D_, nqd, B, db->row_ptr, db->col, db->val, db->sweep, n, false,
+            EMD_CUDA(launch_fwd_b(meas, D_, nqd, B, db->row_ptr, db->col, db->val, db->sweep, n, dir == EMD_DIR_FWD,
                                   table_group(db, ws, meas, tk_b, B), tk_b, st, db->tune_fwd),
                      "forward pass");
+        }
+        if (!pruned) {  // forward direction alone
+            {
+                Phase p(db, 6, 1, st);
+                EMD_CUDA(launch_qpos_b(D_, nqd, B, db->vslot, db->v, false, st), "identical ids");
+            }
+            if (K > 0) {
+                Phase p(db, 5, topk_launch_count(n), st);
+                EMD_CUDA(launch_topk_b(D_, nqd, B, n, K, ws.topk_scratch, false, st), "top-K");
+            }
+            return EMD_OK;
         }
         {
             Phase p(db, 5, topk_launch_count(n), st);
