@@ -452,9 +452,10 @@ __global__ void k_rev_generic(const int32_t* __restrict__ row_ptr, const int32_t
 //
 // Keys are (float bits of the distance << 32) | document id: distances are >= 0, so the
 // unsigned order of the keys is the (distance, id) order and every key is unique.
-// Each thread keeps a sorted register list of its KT smallest keys; the block merges the
-// lists pairwise in shared memory (log2(threads) levels).  With several blocks per query
-// the block results go to scratch and one more block merges them.
+// K <= 32: block_select below.  Beyond, each thread keeps a sorted register list of its KT
+// smallest keys and the block merges the lists pairwise in shared memory (log2(threads)
+// levels).  With several blocks per query the block results go to scratch and one more block
+// merges them.
 
 template <int KT>
 __device__ __forceinline__ void list_insert(unsigned long long (&L)[KT], unsigned long long key)
@@ -506,11 +507,114 @@ __device__ void block_merge_and_emit(unsigned long long (&L)[KT], int K, unsigne
     }
 }
 
+// The K <= 32 smallest keys of a block's range, in two reads of it (the second from cache): the
+// K-th smallest of a warp's 32 lane minima bounds the K-th smallest value of the range, the
+// least bound over the warps leaves about a hundred candidates, and each candidate's rank among
+// them is its place.  Sorted per-thread lists (128 threads, K = 16) spent most of their time on
+// insertions and on a merge of 7 dependent levels: 2e4 values 12.0 + 9.0 -> 4.8 + 3.0 us for the
+// two launches, 64 rows of 1e6 values 437 -> 108 us (their read at HBM rate: 38 us).  Keys are unique; ~0 marks an absent one.  More candidates
+// than slots (many equal values): K rounds of block-wide minima.
+constexpr int kSelThreads = 256, kSelCap = 1024;
+
+template <class F>
+__device__ __forceinline__ void block_select(F key_at, int64_t lo, int64_t hi, int K, int slots,
+                                             unsigned long long* out_keys, int64_t* out_idx, float* out_dist)
+{
+    __shared__ unsigned long long cand[kSelCap];
+    __shared__ unsigned bound[kSelThreads / 32];
+    __shared__ int cnt;
+    const int tid = threadIdx.x, lane = tid & 31;
+    auto emit = [&](int r, unsigned long long key) {
+        if (out_keys) out_keys[r] = key;
+        if (out_idx) {
+            out_idx[r] = (key == ~0ull) ? -1 : (int64_t)(key & 0xffffffffull);
+            out_dist[r] = (key == ~0ull) ? INFINITY : __uint_as_float((unsigned)(key >> 32));
+        }
+    };
+    unsigned m = ~0u;
+#pragma unroll 4
+    for (int64_t i = lo + tid; i < hi; i += kSelThreads) m = min(m, (unsigned)(key_at(i) >> 32));
+#pragma unroll
+    for (int w = 2; w <= 32; w <<= 1) {  // bitonic sort of the lane minima
+#pragma unroll
+        for (int j = w >> 1; j > 0; j >>= 1) {
+            const unsigned o = __shfl_xor_sync(0xffffffffu, m, j);
+            const bool keep_min = ((lane & j) == 0) == ((lane & w) == 0);
+            m = keep_min ? min(m, o) : max(m, o);
+        }
+    }
+    m = __shfl_sync(0xffffffffu, m, K - 1);
+    if (lane == 0) bound[tid >> 5] = m;
+    if (tid == 0) cnt = 0;
+    __syncthreads();
+    unsigned T = bound[0];
+#pragma unroll
+    for (int w = 1; w < kSelThreads / 32; ++w) T = min(T, bound[w]);
+#pragma unroll 4
+    for (int64_t i = lo + tid; i < hi; i += kSelThreads) {
+        const unsigned long long key = key_at(i);
+        if ((unsigned)(key >> 32) <= T && key != ~0ull) {
+            const int p = atomicAdd(&cnt, 1);
+            if (p < kSelCap) cand[p] = key;
+        }
+    }
+    __syncthreads();
+    const int c = cnt;
+    if (c <= kSelCap) {
+        for (int i = tid; i < c; i += kSelThreads) {
+            const unsigned long long me = cand[i];
+            int r = 0;
+            for (int j = 0; j < c; ++j) r += cand[j] < me ? 1 : 0;
+            if (r < K) emit(r, me);
+        }
+        for (int r = min(c, K) + tid; r < slots; r += kSelThreads) emit(r, ~0ull);
+        return;
+    }
+    unsigned long long last = 0;
+    for (int r = 0; r < K; ++r) {
+        unsigned long long best = ~0ull;
+        for (int64_t i = lo + tid; i < hi; i += kSelThreads) {
+            const unsigned long long key = key_at(i);
+            if ((r == 0 || key > last) && key < best) best = key;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long b = __shfl_xor_sync(0xffffffffu, best, o);
+            best = b < best ? b : best;
+        }
+        __syncthreads();
+        if (lane == 0) cand[tid >> 5] = best;
+        __syncthreads();
+        best = cand[0];
+        for (int w = 1; w < kSelThreads / 32; ++w) best = cand[w] < best ? cand[w] : best;
+        last = best;
+        if (tid == 0) emit(r, best);
+    }
+    for (int r = K + tid; r < slots; r += kSelThreads) emit(r, ~0ull);
+}
+
+__device__ __forceinline__ unsigned long long topk_key(float v, int64_t i)
+{
+    return ((unsigned long long)__float_as_uint(v) << 32) | (unsigned long long)(uint32_t)i;
+}
+
+// Threads of the selection kernels for list width KT (the wide form keeps the sorted lists).
+constexpr int topk_threads(int KT) { return KT <= 32 ? kSelThreads : kTopkThreads; }
+
 template <int KT>
 __device__ __forceinline__ void topk_values_body(const float* __restrict__ t, int64_t n, int K, int64_t per_block,
                                                  unsigned long long* __restrict__ scratch_row,
                                                  int64_t* __restrict__ out_idx, float* __restrict__ out_dist)
 {
+    if constexpr (KT <= 32) {
+        const int64_t a = (int64_t)blockIdx.x * per_block, b = min(n, a + per_block);
+        auto key_at = [&](int64_t i) { return topk_key(t[i], i); };
+        if (gridDim.x == 1)
+            block_select(key_at, a, b, K, K, nullptr, out_idx, out_dist);
+        else
+            block_select(key_at, a, b, K, KT, scratch_row + (int64_t)blockIdx.x * KT, nullptr, nullptr);
+        return;
+    }
     unsigned long long L[KT];
 #pragma unroll
     for (int l = 0; l < KT; ++l) L[l] = ~0ull;
@@ -531,6 +635,10 @@ template <int KT>
 __device__ __forceinline__ void topk_keys_body(const unsigned long long* __restrict__ keys, int64_t count, int K,
                                                int64_t* __restrict__ out_idx, float* __restrict__ out_dist)
 {
+    if constexpr (KT <= 32) {
+        block_select([&](int64_t i) { return keys[i]; }, 0, count, K, K, nullptr, out_idx, out_dist);
+        return;
+    }
     unsigned long long L[KT];
 #pragma unroll
     for (int l = 0; l < KT; ++l) L[l] = ~0ull;
@@ -539,7 +647,7 @@ __device__ __forceinline__ void topk_keys_body(const unsigned long long* __restr
 }
 
 template <int KT>
-__global__ void __launch_bounds__(kTopkThreads)
+__global__ void __launch_bounds__(topk_threads(KT))
 k_topk_values(const float* __restrict__ t, int64_t n, int64_t ldt, int K, int64_t per_block,
               unsigned long long* __restrict__ scratch, int64_t* __restrict__ out_idx,
               float* __restrict__ out_dist)
@@ -550,7 +658,7 @@ k_topk_values(const float* __restrict__ t, int64_t n, int64_t ldt, int K, int64_
 }
 
 template <int KT>
-__global__ void __launch_bounds__(kTopkThreads)
+__global__ void __launch_bounds__(topk_threads(KT))
 k_topk_keys(const unsigned long long* __restrict__ keys, int64_t count, int K,
             int64_t* __restrict__ out_idx, float* __restrict__ out_dist)
 {
@@ -561,7 +669,7 @@ k_topk_keys(const unsigned long long* __restrict__ keys, int64_t count, int K,
 // Batched forms: row q of the batch reads qd[q].t_fwd and writes sel_idx / sel_val (the
 // forward top-K of the pruned path, fwd_rows) or reads t_out and writes out_idx / out_dist.
 template <int KT>
-__global__ void __launch_bounds__(kTopkThreads)
+__global__ void __launch_bounds__(topk_threads(KT))
 k_topk_values_b(const QDesc* __restrict__ qd, const int* __restrict__ nq, int64_t n, int K, int64_t per_block,
                 unsigned long long* __restrict__ scratch, bool fwd_rows, bool uncertified)
 {
@@ -574,7 +682,7 @@ k_topk_values_b(const QDesc* __restrict__ qd, const int* __restrict__ nq, int64_
 }
 
 template <int KT>
-__global__ void __launch_bounds__(kTopkThreads)
+__global__ void __launch_bounds__(topk_threads(KT))
 k_topk_keys_b(const QDesc* __restrict__ qd, const int* __restrict__ nq, int64_t count, int K,
               const unsigned long long* __restrict__ scratch, bool fwd_rows, bool uncertified)
 {
@@ -589,17 +697,17 @@ template <int KT>
 cudaError_t topk_kt_b(const QDesc* qd, const int* nq, int max_q, int64_t n, int K, unsigned long long* scratch,
                       bool fwd_rows, bool uncertified, cudaStream_t st)
 {
-    const size_t smem = (size_t)kTopkThreads * KT * sizeof(unsigned long long);
+    const size_t smem = KT <= 32 ? 0 : (size_t)kTopkThreads * KT * sizeof(unsigned long long);
     const int blocks = topk_blocks(n);
     const int64_t per_block = (n + blocks - 1) / blocks;
     if (smem > 48 * 1024) {
         cudaFuncSetAttribute(k_topk_values_b<KT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         cudaFuncSetAttribute(k_topk_keys_b<KT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     }
-    k_topk_values_b<KT><<<dim3(blocks, (unsigned)max_q), kTopkThreads, smem, st>>>(qd, nq, n, K, per_block, scratch,
+    k_topk_values_b<KT><<<dim3(blocks, (unsigned)max_q), topk_threads(KT), smem, st>>>(qd, nq, n, K, per_block, scratch,
                                                                                     fwd_rows, uncertified);
     if (blocks > 1)
-        k_topk_keys_b<KT><<<(unsigned)max_q, kTopkThreads, smem, st>>>(qd, nq, (int64_t)blocks * KT, K, scratch,
+        k_topk_keys_b<KT><<<(unsigned)max_q, topk_threads(KT), smem, st>>>(qd, nq, (int64_t)blocks * KT, K, scratch,
                                                                         fwd_rows, uncertified);
     return cudaGetLastError();
 }
@@ -608,17 +716,17 @@ template <int KT>
 cudaError_t topk_kt(const float* t, int64_t rows, int64_t n, int64_t ldt, int K,
                     unsigned long long* scratch, int64_t* out_idx, float* out_dist, cudaStream_t st)
 {
-    const size_t smem = (size_t)kTopkThreads * KT * sizeof(unsigned long long);
+    const size_t smem = KT <= 32 ? 0 : (size_t)kTopkThreads * KT * sizeof(unsigned long long);
     const int blocks = topk_blocks(n);
     const int64_t per_block = (n + blocks - 1) / blocks;
     if (smem > 48 * 1024) {
         cudaFuncSetAttribute(k_topk_values<KT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         cudaFuncSetAttribute(k_topk_keys<KT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     }
-    k_topk_values<KT><<<dim3(blocks, (unsigned)rows), kTopkThreads, smem, st>>>(t, n, ldt, K, per_block, scratch,
+    k_topk_values<KT><<<dim3(blocks, (unsigned)rows), topk_threads(KT), smem, st>>>(t, n, ldt, K, per_block, scratch,
                                                                                  out_idx, out_dist);
     if (blocks > 1)
-        k_topk_keys<KT><<<(unsigned)rows, kTopkThreads, smem, st>>>(scratch, (int64_t)blocks * KT, K, out_idx,
+        k_topk_keys<KT><<<(unsigned)rows, topk_threads(KT), smem, st>>>(scratch, (int64_t)blocks * KT, K, out_idx,
                                                                      out_dist);
     return cudaGetLastError();
 }
