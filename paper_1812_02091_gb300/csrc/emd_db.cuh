@@ -149,6 +149,10 @@ struct emd_db {
     int32_t* used_ids = nullptr; // v_used, vocabulary id of each used row (ascending)
     float* cost = nullptr;       // v x v ground costs (cost-matrix mode)
     int32_t* row_ptr = nullptr;  // n + 1
+    // host check of repeated query ids: the last check that met each vocabulary id, and the number of
+    // the current one (both under mu)
+    std::vector<int64_t> q_seen;
+    int64_t q_check = 0;
     std::vector<int64_t> row_ptr_host;  // the same offsets on the host (all-pairs batching)
     int32_t* col = nullptr;      // nnz, renumbered into the used vocabulary
     float* val = nullptr;        // nnz
@@ -270,7 +274,7 @@ struct Phase {
 int table_width(const emd_db* db, int meas, int k, int h);
 // Candidates per row re-ranked by the table kernel of the approximate precisions.
 int rerank_width(const emd_db* db, int tk, int h);
-emd_status check_query_values(const emd_db* db, const emd_queries* q);
+emd_status check_query_values(emd_db* db, const emd_queries* q);  // caller holds db->mu
 bool prunable(const emd_db* db, int meas, int k, int dir, int K);
 int topk_launch_count(int64_t n);
 
