@@ -541,6 +541,23 @@ __device__ __forceinline__ void table_rerank_body(float* __restrict__ D, int ldd
             }
         }
     }
+    // The order of the candidates is free (sums are per candidate, the final list is by value and bin):
+    // ordered by their bank group from the lane's own on, the eight lanes of a shared-memory
+    // phase tend to read different groups (the L1 data path is 80% busy with these reads).  41 queries of
+    // 20..400 bins, 93,255 words, k = 2: 5.03 -> 4.96 ms.
+#pragma unroll
+    for (int c = 0; c < KCT; ++c)
+        if (c >= kc) s[c] = INT32_MAX;
+#pragma unroll
+    for (int a = 0; a < KCT; ++a) {
+#pragma unroll
+        for (int c = a & 1; c + 1 < KCT; c += 2) {
+            const int p = s[c], q = s[c + 1];
+            const int kp = p == INT32_MAX ? 8 : (p - tid) & 7, kq = q == INT32_MAX ? 8 : (q - tid) & 7;
+            s[c] = kq < kp ? q : p;
+            s[c + 1] = kq < kp ? p : q;
+        }
+    }
     float acc[KCT];
 #pragma unroll
     for (int l = 0; l < KCT; ++l) acc[l] = 0.f;
