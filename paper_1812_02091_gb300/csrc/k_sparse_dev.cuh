@@ -507,13 +507,19 @@ __device__ void block_merge_and_emit(unsigned long long (&L)[KT], int K, unsigne
     }
 }
 
-// The K <= 32 smallest keys of a block's range, in two reads of it (the second from cache): the
-// K-th smallest of a warp's 32 lane minima bounds the K-th smallest value of the range, the
-// least bound over the warps leaves about a hundred candidates, and each candidate's rank among
-// them is its place.  Sorted per-thread lists (128 threads, K = 16) spent most of their time on
-// insertions and on a merge of 7 dependent levels: 2e4 values 12.0 + 9.0 -> 4.8 + 3.0 us for the
-// two launches, 64 rows of 1e6 values 437 -> 108 us (their read at HBM rate: 38 us).  Keys are unique; ~0 marks an absent one.  More candidates
-// than slots (many equal values): K rounds of block-wide minima.
+// The K <= 32 smallest keys of a block's range, in two reads of it (the second from cache): a bound
+// on the K-th smallest key from the 256 lane minima leaves some tens of candidates, and each
+// candidate's rank among them is its place.  Two bounds hold, and the smaller one counts: the K-th
+// smallest minimum of one warp (rows in order, small ranges), and the largest over the 8 warps of
+// each one's ceil(K / 8)-th smallest (values in any order; the first alone lets 640 through at K = 32).
+// The minima are whole keys, value and id: with the value alone, rows of equal values -- duplicate
+// documents, the second stage's rows of +inf -- let every key through.
+// 64 rows of 1e6 values (256 MB, 38 us at HBM rate), K = 16: 91 us for random values, 89 us with
+// 100 finite values a row, 88 us all equal (103, 685 and 685 us by the values of one warp's minima,
+// 463, 206 and 208 us by sorted per-thread lists); K = 32: 98, 93 and 90 us (382, 1181 and 1182 us; 928,
+// 549 and 551 us).  One row of 2e4 values, K = 16, both launches: 17 us (17; 29 us).
+// Keys are unique; ~0 marks an absent one.  More candidates than slots takes hundreds of small
+// values in few of the lanes (every 256th place): K rounds of block-wide minima.
 constexpr int kSelThreads = 256, kSelCap = 1024;
 
 template <class F>
@@ -521,7 +527,7 @@ __device__ __forceinline__ void block_select(F key_at, int64_t lo, int64_t hi, i
                                              unsigned long long* out_keys, int64_t* out_idx, float* out_dist)
 {
     __shared__ unsigned long long cand[kSelCap];
-    __shared__ unsigned bound[kSelThreads / 32];
+    __shared__ unsigned long long bound[kSelThreads / 32], share[kSelThreads / 32];
     __shared__ int cnt;
     const int tid = threadIdx.x, lane = tid & 31;
     auto emit = [&](int r, unsigned long long key) {
@@ -531,29 +537,41 @@ __device__ __forceinline__ void block_select(F key_at, int64_t lo, int64_t hi, i
             out_dist[r] = (key == ~0ull) ? INFINITY : __uint_as_float((unsigned)(key >> 32));
         }
     };
-    unsigned m = ~0u;
+    constexpr int W = kSelThreads / 32;
+    unsigned long long m = ~0ull;
 #pragma unroll 4
-    for (int64_t i = lo + tid; i < hi; i += kSelThreads) m = min(m, (unsigned)(key_at(i) >> 32));
+    for (int64_t i = lo + tid; i < hi; i += kSelThreads) {
+        const unsigned long long key = key_at(i);
+        m = key < m ? key : m;
+    }
 #pragma unroll
     for (int w = 2; w <= 32; w <<= 1) {  // bitonic sort of the lane minima
 #pragma unroll
         for (int j = w >> 1; j > 0; j >>= 1) {
-            const unsigned o = __shfl_xor_sync(0xffffffffu, m, j);
+            const unsigned long long o = __shfl_xor_sync(0xffffffffu, m, j);
             const bool keep_min = ((lane & j) == 0) == ((lane & w) == 0);
-            m = keep_min ? min(m, o) : max(m, o);
+            m = (o < m) == keep_min ? o : m;
         }
     }
-    m = __shfl_sync(0xffffffffu, m, K - 1);
-    if (lane == 0) bound[tid >> 5] = m;
+    const unsigned long long all = __shfl_sync(0xffffffffu, m, K - 1);
+    const unsigned long long part = __shfl_sync(0xffffffffu, m, (K + W - 1) / W - 1);
+    if (lane == 0) {
+        bound[tid >> 5] = all;
+        share[tid >> 5] = part;
+    }
     if (tid == 0) cnt = 0;
     __syncthreads();
-    unsigned T = bound[0];
+    unsigned long long T = bound[0], S = share[0];
 #pragma unroll
-    for (int w = 1; w < kSelThreads / 32; ++w) T = min(T, bound[w]);
+    for (int w = 1; w < W; ++w) {
+        T = bound[w] < T ? bound[w] : T;
+        S = share[w] > S ? share[w] : S;
+    }
+    T = S < T ? S : T;
 #pragma unroll 4
     for (int64_t i = lo + tid; i < hi; i += kSelThreads) {
         const unsigned long long key = key_at(i);
-        if ((unsigned)(key >> 32) <= T && key != ~0ull) {
+        if (key <= T && key != ~0ull) {
             const int p = atomicAdd(&cnt, 1);
             if (p < kSelCap) cand[p] = key;
         }
