@@ -218,8 +218,16 @@ __device__ __forceinline__ void rev_body(const int32_t* __restrict__ row_ptr, co
     }
 }
 
+// Resident blocks per SM of the passes over documents.  Lists of one or two entries fit 64 registers;
+// left to themselves the narrower passes take 66 to 74 and cost RWMD and one-entry ACT the fourth
+// block.  Wider lists take 80 registers and three blocks (two: 8% slower at k = 4 and 8).  32 queries
+// of 40 .. 260 bins, 2e4 documents, at 3 and 4 blocks: RWMD 3.33 and 2.73 ms, OMR 4.85 and 4.56, ACT k = 1
+// 3.87 and 3.46 (3.17, 6.01 and 4.23 before the narrower passes); 8 queries of 150 bins one by one,
+// k = 2: 2.48 and 2.35 ms.
+constexpr int rev_blocks(int kt) { return kt <= 2 ? 4 : 3; }
+
 template <int MEAS, int KT, int NJ>
-__global__ void __launch_bounds__(256, 3) k_rev(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
+__global__ void __launch_bounds__(256, rev_blocks(KT)) k_rev(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col,
       const float* __restrict__ val, int64_t n, const float* __restrict__ D, int ldd, int h,
       const float* __restrict__ q_w, int k, const float* __restrict__ t_fwd,
       float* __restrict__ t_rev, float* __restrict__ t_max, const int64_t* __restrict__ doc_ids,
@@ -848,7 +856,7 @@ cudaError_t rev_meas_blk(int k, const int32_t* row_ptr, const int32_t* col, cons
 
 // NJ follows the per-query launcher: NJW bins per lane when h > 32, else one.
 template <int MEAS, int KT, int NJW>
-__global__ void __launch_bounds__(256, 3)
+__global__ void __launch_bounds__(256, rev_blocks(KT))
 k_rev_b(const QDesc* __restrict__ qd, const int* __restrict__ nq, const int32_t* __restrict__ row_ptr,
         const int32_t* __restrict__ col, const float* __restrict__ val, int64_t n, int k, int dir)
 {
@@ -954,7 +962,7 @@ cudaError_t rev_meas_b(int k, int dir, const QDesc* qd, const int* nq, int max_q
 // documents took 3.3 ms a query on 60,000 images (k = 8, top-16: 25 to 32 queries of a batch
 // of 64 are not certified); this takes 106 ms per batch to 2.3 ms.
 template <int MEAS, int KT, int NJW>
-__global__ void __launch_bounds__(256, 3)
+__global__ void __launch_bounds__(256, rev_blocks(KT))
 k_rev_within_b(const QDesc* __restrict__ qd, const int* __restrict__ nq, const int32_t* __restrict__ row_ptr,
                const int32_t* __restrict__ col, const float* __restrict__ val, int64_t n, int k, int K)
 {
