@@ -10,7 +10,7 @@ import pytest
 
 from paper_1812_02091_gb300 import _build
 
-SOURCES = ("k_sparse.cu", "k_sparse_b.cu", "k_within_b.cu")
+SOURCES = ("k_phase1.cu", "k_sparse.cu", "k_sparse_b.cu", "k_within_b.cu")
 
 
 def _compile(source):
@@ -34,3 +34,9 @@ def kernels():
 def test_blocks_per_sm(kernels, source, kernel, registers):
     found = {n: r for n, (r, _) in kernels[source].items() if re.search(kernel, n)}
     assert found and max(found.values()) <= registers, found
+
+
+@pytest.mark.parametrize("kernel", [r"k_dist_fp32E", r"k_dist_fp32_bE"])
+def test_no_spills(kernels, kernel):
+    found = {n: b for n, (_, b) in kernels["k_phase1.cu"].items() if re.search(kernel, n)}
+    assert len(found) == 1 and not any(found.values()), found
