@@ -552,13 +552,13 @@ emd_status launch_sequence(BatchWS& ws, emd_db* db, int slot, int meas, int k, i
 // Captures launch_sequence for these parameters into an executable graph (on the handle's
 // capture stream); the launch counts of one replay are kept beside it.
 emd_status capture_sequence(BatchWS& ws, emd_db* db, int slot, int meas, int k, int K, int dir, bool pruned, int qcap,
-                            GraphEntry* g, bool allow_fused)
+                            GraphEntry* g)
 {
     int64_t l0[EMD_N_PHASES], t0 = db->total_launches;
     for (int p = 0; p < EMD_N_PHASES; ++p) l0[p] = db->launches[p];
     cudaStream_t cs = ws.cap_stream;
     EMD_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal), "graph capture");
-    emd_status s = launch_sequence(ws, db, slot, meas, k, K, dir, pruned, nullptr, 0, qcap, cs, allow_fused);
+    emd_status s = launch_sequence(ws, db, slot, meas, k, K, dir, pruned, nullptr, 0, qcap, cs);
     cudaGraph_t graph = nullptr;
     const cudaError_t e = cudaStreamEndCapture(cs, &graph);
     for (int p = 0; p < EMD_N_PHASES; ++p) {
@@ -825,20 +825,22 @@ emd_status run_subbatch_launch(BatchWS& ws, int slot, emd_db* db, int nb, int me
         // embeddings too wide for the batched panel: Phase 1 per query, the rest batched
         return launch_sequence(ws, db, slot, meas, k, K, dir, pruned, hd, nb, qcap, st);
     }
-    if (!db->opt.graphs || db->profiling)
+    // reruns of uncertified queries (the only calls that rule the fused form out) are launched directly:
+    // a graph per ring slot and size class would be captured for sequences that rarely come again
+    if (!db->opt.graphs || db->profiling || !allow_fused)
         return launch_sequence(ws, db, slot, meas, k, K, dir, pruned, nullptr, 0, qcap, st, allow_fused);
-    const GraphKey key{meas, k, K, dir, pruned ? 1 : 0, slot, qcap, allow_fused ? 1 : 0};
+    const GraphKey key{meas, k, K, dir, pruned ? 1 : 0, slot, qcap};
     auto it = ws.graphs.find(key);
     if (it == ws.graphs.end()) {
         GraphEntry g;
-        emd_status cs = capture_sequence(ws, db, slot, meas, k, K, dir, pruned, qcap, &g, allow_fused);
+        emd_status cs = capture_sequence(ws, db, slot, meas, k, K, dir, pruned, qcap, &g);
         if (cs != EMD_OK) {
             g_err.clear();
             g.exec = nullptr;  // capture refused: this key launches directly from now on
         }
         it = ws.graphs.emplace(key, g).first;
     }
-    if (!it->second.exec) return launch_sequence(ws, db, slot, meas, k, K, dir, pruned, nullptr, 0, qcap, st, allow_fused);
+    if (!it->second.exec) return launch_sequence(ws, db, slot, meas, k, K, dir, pruned, nullptr, 0, qcap, st);
     EMD_CUDA(cudaGraphLaunch(it->second.exec, st), "graph launch");
     for (int p = 0; p < EMD_N_PHASES; ++p) db->launches[p] += it->second.launches[p];
     db->total_launches += it->second.total;

@@ -51,10 +51,8 @@ namespace emd {
 // One captured batch sequence (launch_sequence) and the kernel launches it holds.
 struct GraphKey {
     int meas, k, K, dir, pruned, slot, qcap;  // qcap: queries the grids cover (power of two)
-    int fused;                                // fused pruned path allowed
     bool operator<(const GraphKey& o) const
     {
-        if (fused != o.fused) return fused < o.fused;
         if (meas != o.meas) return meas < o.meas;
         if (k != o.k) return k < o.k;
         if (K != o.K) return K < o.K;
