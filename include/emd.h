@@ -124,7 +124,7 @@ typedef struct {
                                 table rows, four entries loaded up front; 3 the first two entries up
                                 front, column ids and weights read 32 at a time; 4 as 1 with each
                                 lane's next column ids and weights read ahead.  Same results */
-    int32_t tc_pair;         /* the fused FP32_TC table (fused_phase1 >= 1) on clusters of two SMs
+    int32_t tc_pair;         /* the pruned top-K's fused FP32_TC table (fused_phase1 >= 1) on clusters of two SMs
                                 (tcgen05 cta_group::2: 256 vocabulary rows per product, each SM
                                 staging half of each query chunk): 0 (default) one SM per tile;
                                 1 pairs with 64-column tiles; 2 pairs with 128-column tiles.

@@ -98,7 +98,7 @@ cudaEvent_t take_event(emd_db* db)
     return e;
 }
 
-// The fused FP32_TC table runs on SM pairs when the option asks for it and the panel fits.
+// The pruned top-K's fused FP32_TC table runs on SM pairs when the option asks for it and the panel fits.
 bool use_tc_pair(const emd_db* db)
 {
     return db->opt.tc_pair > 0 && db->tc && db->tcfmt == TC_SPLIT && !db->cost_mode && db->mpad % 256 == 0 &&
@@ -401,7 +401,9 @@ emd_status launch_sequence(BatchWS& ws, emd_db* db, int slot, int meas, int k, i
         {
             Phase p(db, 1, 2, st);
             EMD_CUDA(launch_qpos_b(D_, nqd, B, db->vslot, db->v, true, st), "identical ids");
-            if (use_tc_pair(db))
+            // SM pairs for the pruned top-K alone: the forward direction's other calls never ran on them, and with
+            // 64-column tiles they are slower than the matrix (20 queries, 3e4 words: 0.56 against 0.51 ms; one SM 0.46)
+            if (pruned && use_tc_pair(db))
                 EMD_CUDA(launch_tc_table_pair(db->a_hi, db->a_lo, db->mpad, db->a_scale, db->norm_used, db->v_used,
                                               D_, nqd, B, db->kpad, db->m, tk_b, db->tune_group_mult,
                                               db->opt.tc_pair == 1 ? 64 : 128, db->err, st),
