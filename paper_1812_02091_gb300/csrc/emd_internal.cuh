@@ -22,29 +22,13 @@ enum : int { M_RWMD = 0, M_OMR = 1, M_ACT = 2, M_ICT = 3 };
 __device__ __forceinline__ float sq_to_dist(float x) { return __fsqrt_rn(fmaxf(x, 0.f)); }
 __device__ __forceinline__ float d_value(float x, bool sq) { return sq ? sq_to_dist(x) : x; }
 
-// Two FP32 operations in one instruction, each rounded as its scalar form.
+// Two FP32 fused multiply-adds in one instruction, each rounded as fmaf.
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
 {
     float2 d;
     asm("fma.rn.f32x2 %0, %1, %2, %3;"
         : "=l"(reinterpret_cast<uint64_t&>(d))
         : "l"(reinterpret_cast<uint64_t&>(a)), "l"(reinterpret_cast<uint64_t&>(b)), "l"(reinterpret_cast<uint64_t&>(c)));
-    return d;
-}
-__device__ __forceinline__ float2 mul2(float2 a, float2 b)
-{
-    float2 d;
-    asm("mul.rn.f32x2 %0, %1, %2;"
-        : "=l"(reinterpret_cast<uint64_t&>(d))
-        : "l"(reinterpret_cast<uint64_t&>(a)), "l"(reinterpret_cast<uint64_t&>(b)));
-    return d;
-}
-__device__ __forceinline__ float2 add2(float2 a, float2 b)
-{
-    float2 d;
-    asm("add.rn.f32x2 %0, %1, %2;"
-        : "=l"(reinterpret_cast<uint64_t&>(d))
-        : "l"(reinterpret_cast<uint64_t&>(a)), "l"(reinterpret_cast<uint64_t&>(b)));
     return d;
 }
 

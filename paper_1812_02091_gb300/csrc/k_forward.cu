@@ -568,27 +568,26 @@ cudaError_t launch_interleave(const int32_t* col, const float* val, int64_t nnz,
 }
 
 template <int G>
-static void fwd_chain(int m, int kw, int max_tk, const QDesc* qd, const int* nq, int max_q, const int32_t* row_ptr,
-                      const FwdSweep& w, int64_t n, bool to_out, cudaStream_t st)
+static cudaError_t fwd_chain(int m, int kw, int max_tk, const QDesc* qd, const int* nq, int max_q, const int32_t* row_ptr,
+                             const FwdSweep& w, int64_t n, bool to_out, cudaStream_t st)
 {
     constexpr int warps = kFwdThreads / 32;
     // documents per warp: one, or for large databases four (fewer block launches)
     const int per_warp = n > 200000 ? 4 : 1;
     const dim3 gg((unsigned)((n + w.n_long + warps * per_warp - 1) / (warps * per_warp)), (unsigned)((max_q + G - 1) / G));
 #define EMD_LM(M, KT) k_fwd_g<M, KT, G, fwd_un(M, KT, G)><<<gg, kFwdThreads, 0, st>>>(qd, nq, row_ptr, w.cv, n, w.long_docs, w.n_long, w.long_len, per_warp, to_out)
-    switch (m) {
-    case M_RWMD: EMD_LM(M_RWMD, 0); break;
-    case M_OMR:
-        if (max_tk >= 2) EMD_LM(M_OMR, 0); else EMD_LM(M_RWMD, 0);  // one-bin queries: tables of one entry, same cost
-        break;
-    default: {
+    // tables of one entry: RWMD's, and OMR's when every query has one bin (the same cost)
+    if (m == M_RWMD || (m == M_OMR && max_tk < 2)) EMD_LM(M_RWMD, 0);
+    else if (m == M_ACT && kw == 1) EMD_LM(M_ACT, 1);
+    else if constexpr (G == 16) return cudaErrorInvalidValue;  // fwd_chain_group: 16 queries for one entry only
+    else if (m == M_OMR) EMD_LM(M_OMR, 0);
+    else {
 #define EMD_L(KT) EMD_LM(M_ACT, KT)
         EMD_FWD_KT_SWITCH(kw, EMD_L)
 #undef EMD_L
-        break;
-    }
     }
 #undef EMD_LM
+    return cudaGetLastError();
 }
 
 cudaError_t launch_fwd_b(int meas, const QDesc* qd, const int* nq, int max_q, const int32_t* row_ptr,
@@ -618,14 +617,13 @@ cudaError_t launch_fwd_b(int meas, const QDesc* qd, const int* nq, int max_q, co
         }
         if (kw == 0 || variant == kFwdChain) {  // entry-interleaved rows, loads while mass remains
             switch (group) {
-            case 1: fwd_chain<1>(m, kw, max_tk, qd, nq, max_q, row_ptr, sweep, n, to_out, st); break;
-            case 2: fwd_chain<2>(m, kw, max_tk, qd, nq, max_q, row_ptr, sweep, n, to_out, st); break;
-            case 4: fwd_chain<4>(m, kw, max_tk, qd, nq, max_q, row_ptr, sweep, n, to_out, st); break;
-            case 8: fwd_chain<8>(m, kw, max_tk, qd, nq, max_q, row_ptr, sweep, n, to_out, st); break;
-            case 16: fwd_chain<16>(m, kw, max_tk, qd, nq, max_q, row_ptr, sweep, n, to_out, st); break;
+            case 1: return fwd_chain<1>(m, kw, max_tk, qd, nq, max_q, row_ptr, sweep, n, to_out, st);
+            case 2: return fwd_chain<2>(m, kw, max_tk, qd, nq, max_q, row_ptr, sweep, n, to_out, st);
+            case 4: return fwd_chain<4>(m, kw, max_tk, qd, nq, max_q, row_ptr, sweep, n, to_out, st);
+            case 8: return fwd_chain<8>(m, kw, max_tk, qd, nq, max_q, row_ptr, sweep, n, to_out, st);
+            case 16: return fwd_chain<16>(m, kw, max_tk, qd, nq, max_q, row_ptr, sweep, n, to_out, st);
             default: return cudaErrorInvalidValue;
             }
-            return cudaGetLastError();
         }
 #define EMD_GV(M, KT)                                                                                       \
     do {                                                                                                    \
