@@ -120,8 +120,9 @@ __global__ void k_fwd(const int32_t* __restrict__ row_ptr, const int32_t* __rest
 // resident blocks per SM (the register bound).  Groups of up to 4 queries have few warps to
 // run and take more nonzeros each; paired tables at 32 blocks (all 64 warps) and two
 // nonzeros beat 16 to 24 blocks with up to four (serving database, 64 queries: 9.9 against
-// 10.5 to 13.1 ms, a few spilled registers included); single-entry tables are fastest at 24
-// blocks and three.
+// 10.5 to 13.1 ms, a few spilled registers included); single-entry tables are faster at 24
+// blocks and three than at 32 and two (64 queries, 1e6 documents: 9.8 against 11.5 ms, 2e4: 0.237
+// against 0.269).
 constexpr int kFwdThreads = 64;
 constexpr int fwd_un(int meas, int kt, int g) { return g <= 4 ? 4 : meas == M_RWMD || kt == 1 ? 3 : 2; }
 constexpr int fwd_blocks(int meas, int kt, int g) { return g <= 4 ? 16 : meas == M_RWMD || kt == 1 ? 24 : 32; }
@@ -572,7 +573,11 @@ static cudaError_t fwd_chain(int m, int kw, int max_tk, const QDesc* qd, const i
                              const FwdSweep& w, int64_t n, bool to_out, cudaStream_t st)
 {
     constexpr int warps = kFwdThreads / 32;
-    // documents per warp: one, or for large databases four (fewer block launches)
+    // documents per warp: one, or for large databases four (fewer block launches).  One and four, ms: 64
+    // queries, k = 4: 1e6 documents 11.04 and 10.28, 250,000 2.72 and 2.54, 1e5 1.11 and 1.06, 2e4 0.228 and
+    // 0.278; k = 1: 10.46 and 9.80, 2.64 and 2.50, 1.09 and 1.06, 0.237 and 0.360; one query: 0.556 and
+    // 0.469, 0.156 and 0.137, 0.071 and 0.066, 0.022 and 0.028.  Four already gains 5% from 1e5 on; the
+    // line keeps clear of the small databases, where whole warps would stay without a document.
     const int per_warp = n > 200000 ? 4 : 1;
     const dim3 gg((unsigned)((n + w.n_long + warps * per_warp - 1) / (warps * per_warp)), (unsigned)((max_q + G - 1) / G));
 #define EMD_LM(M, KT) k_fwd_g<M, KT, G, fwd_un(M, KT, G)><<<gg, kFwdThreads, 0, st>>>(qd, nq, row_ptr, w.cv, n, w.long_docs, w.n_long, w.long_len, per_warp, to_out)
