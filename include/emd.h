@@ -102,7 +102,9 @@ typedef struct {
                                 kernels on a synthetic batch at creation and keeps the fastest
                                 (results do not depend on them); 0: fixed defaults */
     int32_t fused_phase1;    /* batched pruned top-K (EMD_DIR_MAX, K <= 16) with RWMD, OMR or ACT
-                                (k <= 16), tensor-core precisions.  The fused form keeps each row's
+                                (k <= 16), tensor-core precisions; with FP32_TC also the calls of the
+                                forward direction alone (distances, top-K of any K, all pairs), which
+                                need no reverse distances.  The fused form keeps each row's
                                 k smallest distances (FP32_TC) or k + rerank_margin <= 16 smallest
                                 approximate ones (BF16, FP8_E4M3) in the product's epilogue, and
                                 computes the reverse direction's distances only on the candidate
@@ -119,14 +121,16 @@ typedef struct {
                                 form: the wide candidate lists and their FP32 re-rank cost about
                                 what the cheaper product saves) */
     int32_t fwd_kernel;      /* form of the batched forward sweep (Phase 2+3 over the CSR for a
-                                group of eight queries): 0 (default) the autotuner's choice; 1 each
-                                table entry loaded when the residual mass needs it; 2 query-major
-                                table rows, four entries loaded up front; 3 the first two entries up
-                                front, column ids and weights read 32 at a time; 4 as 1 with each
-                                lane's next column ids and weights read ahead.  Same results */
-    int32_t tc_pair;         /* the pruned top-K's fused FP32_TC table (fused_phase1 >= 1) on clusters of two SMs
-                                (tcgen05 cta_group::2: 256 vocabulary rows per product, each SM
-                                staging half of each query chunk): 0 (default) one SM per tile;
+                                group of queries): 0 (default) the autotuner's choice; 1 each
+                                pair of table entries loaded when the residual mass needs it,
+                                groups of 1 to 16 queries by the batch's size (the others: eight);
+                                2 query-major table rows, four entries loaded up front; 3 the first
+                                two entries up front, column ids and weights read 32 at a time; 4
+                                one entry at a time, each lane's next column ids and weights read
+                                ahead.  Same results */
+    int32_t tc_pair;         /* the pruned top-K's fused FP32_TC table (fused_phase1 >= 1) on
+                                clusters of two SMs (tcgen05 cta_group::2: 256 vocabulary rows per
+                                product, each SM staging half of each query chunk): 0 (default) one SM per tile;
                                 1 pairs with 64-column tiles; 2 pairs with 128-column tiles.
                                 Same results */
 } emd_db_options;
@@ -164,7 +168,8 @@ typedef struct {
     int64_t launches[EMD_N_PHASES];
     int64_t total_launches; /* every kernel launch since creation, profiling on or off */
     int64_t pruned_queries; /* max-direction top-K queries answered by the pruned path */
-    int64_t prune_fallbacks; /* of those, queries that needed the second stage (see emd_topk) */
+    int64_t prune_fallbacks; /* of those, queries that needed the second stage, or with batched = 0
+                                all documents (see emd_topk) */
     int64_t graph_launches;  /* batch sequences replayed from captured graphs (their kernels are
                                 included in the launch counts) */
     int64_t ict_wide;        /* ICT queries recomputed with tables of full width h because a
@@ -225,9 +230,9 @@ emd_status emd_query_batch(emd_db* db, const emd_queries* q, emd_measure meas, i
  * within a margin of the K-th smallest forward value (at most 256), and the answer is
  * certified when the K-th symmetric value does not exceed that margin.  For a query that
  * fails the test the K-th symmetric value U found so far still bounds the answer, and a second
- * stage evaluates every document with a forward value <= U.  The result equals the unpruned
- * one.
- *   K         1..min(n_docs, 256)
+ * stage evaluates every document with a forward value <= U (with batched = 0 such a query is
+ * recomputed over all documents).  The result equals the unpruned one.
+ *   K         1..min(n_docs, 64)
  *   out_idx   host int64 [n_queries * K]; out_dist host float [n_queries * K]
  * Otherwise as emd_query_batch. */
 emd_status emd_topk(emd_db* db, const emd_queries* q, emd_measure meas, int32_t k,

@@ -204,8 +204,8 @@ struct QDesc {
     int64_t* out_idx;       // K top-K result
     float* out_dist;
     int h, ldd, qrows, npad, tk, kc;
-    // table layout: entry l of row u at tab[u * tab_rs + tab_entry(d, l)] -- tab_es apart, or (pairs)
-    // two entries adjacent and the pairs tab_es apart
+    // table layout: entry l of row u at tab[u * tab_rs + tab_entry(l, tab_es, tab_pair)] -- entries
+    // tab_es apart, or (pairs) two entries adjacent and the pairs tab_es apart
     int tab_rs, tab_es, tab_pair;
     // fused form of the pruned path (Phase-1 table in the product's epilogue, no full matrix)
     int32_t* qpos;          // v_used: the query bin whose vocabulary id is used row u, else -1
@@ -247,17 +247,17 @@ __device__ __forceinline__ float tab_cap(float w, int l, int tk, int pair)
 constexpr int kCandPerRow = 16;
 
 // Largest number of distinct used rows among the candidate documents of one query in the
-// fused pruned path (their distance block is computed exactly; beyond it the query is
-// recomputed over all documents with the full distance matrix).
+// fused pruned path (their distance block is computed exactly; beyond it the query is run
+// again with the full distance matrix, whose certificate can hold).
 constexpr int kCandRows = 32768;
 
 // Queries whose forward pass shares one sweep of the CSR (batched form).  The entry-chain form
 // (the default) takes 1, 2, 4, 8 or 16 queries a group by the batch's size class, the other
 // forms always kFwdGroup.  Tables are interleaved by entry -- row u, entry l, query g of a group of
 // G at base[(u * width + l) * G + g] -- and in the entry-chain form, from width 2 on, by pairs of
-// entries: base[(u * width + (l & ~1)) * G + 2 g + (l & 1)], width rounded up to even; the query-major form stores tables of width <= 16
-// query-major within a row -- row u, query g, entry l at base[(u * kFwdGroup + g) * W + l]
-// with W the register width of the table (1, 2, 4, 8 or 16).
+// entries: base[(u * width + (l & ~1)) * G + 2 g + (l & 1)], width rounded up to even; the
+// query-major form stores tables of width <= 16 query-major within a row -- row u, query g, entry l
+// at base[(u * kFwdGroup + g) * W + l] with W the register width of the table (1, 2, 4, 8 or 16).
 constexpr int kFwdGroup = 8;
 constexpr int kFwdGroupMax = 16;
 // Group size of the entry-chain form for tables of width tk in a batch whose grids cover qcap

@@ -547,7 +547,8 @@ __device__ __forceinline__ void table_rerank_body(float* __restrict__ D, int ldd
     // The order of the candidates is free (sums are per candidate, the final list is by value and bin):
     // ordered by their bank group from the lane's own on, the eight lanes of a shared-memory
     // phase tend to read different groups (the L1 data path is 80% busy with these reads).  41 queries of
-    // 20..400 bins, 93,255 words, k = 2: 5.03 -> 4.96 ms.
+    // 20..400 bins, 93,255 words, without and with it in turn: k = 2 5.12 and 4.97 ms (whole search 6.67 and
+    // 6.46), k = 8 7.72 and 7.38; 20..60 bins 4.03 and 3.90.
 #pragma unroll
     for (int c = 0; c < KCT; ++c)
         if (c >= kc) s[c] = INT32_MAX;

@@ -820,8 +820,9 @@ __device__ __forceinline__ void prune_select_body(const int64_t* __restrict__ ca
         out_dist[i] = INFINITY;
     }
     __syncthreads();
-    // 1: certified; 0: not certified (recompute over all documents); 2: the candidate
-    // block of the fused path overflowed (retry with the full distance matrix)
+    // 1: certified; 0: not certified (second stage; one query at a time: recomputed over all
+    // documents); 2: the candidate block of the fused path overflowed (run again with the full distance
+    // matrix)
     if (i == 0) *ok = !complete ? 2 : (*count <= cap && c >= K && kth <= prune_theta(sel_val[K - 1])) ? 1 : 0;
 }
 
